@@ -434,6 +434,7 @@ rn_status rn_graph_info(const rn_graph *g, rn_graph_stats *out) {
         if (!g || !out) rn::fail(RN_EINVAL, "null argument");
         *out = g->info;
         out->device_bytes = (uint64_t(g->dev.n) + 1) * 4 + g->dev.arcs * 8 + uint64_t(g->dev.n) * 8 +
+                            (g->dev.ell ? (uint64_t(g->dev.n) + g->dev.nvirt) * 64 : 0) +
                             rn::workspace_bytes(g->ws);
     });
 }

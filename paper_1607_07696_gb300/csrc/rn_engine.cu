@@ -148,6 +148,8 @@ void dpairs_release(rn_dpairs *p) {
     p->n = 0;
 }
 
+static void build_rows(const HostGraph &g, DeviceGraph *d);
+
 void upload_graph(const HostGraph &g, const std::vector<uint32_t> &perm,
                   const std::vector<uint32_t> &iperm, DeviceGraph *out) {
     DeviceGraph d;
@@ -170,6 +172,7 @@ void upload_graph(const HostGraph &g, const std::vector<uint32_t> &perm,
         // a copy from pageable memory may still be in flight when cudaMemcpy returns, and
         // queries run on streams that do not wait for the legacy stream
         RN_CUDA(cudaDeviceSynchronize());
+        build_rows(g, &d);
     } catch (...) {
         free_graph(&d);
         throw;
@@ -180,6 +183,7 @@ void upload_graph(const HostGraph &g, const std::vector<uint32_t> &perm,
 void free_graph(DeviceGraph *g) {
     device_free(g->row_ptr);
     device_free(g->adj);
+    device_free(g->ell);
     device_free(g->perm);
     device_free(g->iperm);
     device_free(g->xy);
@@ -241,6 +245,8 @@ struct Control {
     unsigned long long slot_lanes;  // sum over tiles of slots times the tile's lanes
     uint32_t src_max_ball;          // largest ball of a source the warp search completed
     uint32_t max_seg;               // most pairs one source emitted in the warp search
+    uint32_t src_max_pages;         // most pages of a ball the source search completed
+    unsigned long long pages;       // sum over those balls of their pages
 };
 
 // Record the first failed device-side check (the access it guarded is skipped).
@@ -323,7 +329,7 @@ struct Workspace {
     uint64_t mq_cap_q = 0, mq_cap_bits = 0, mq_cap_sids = 0;
     // the largest source ball the last warp search met (or estimated, for sources
     // whose map overflowed) and its bound: predicts the next query's balls
-    double ball_max = 0, ball_mean = 0;
+    double ball_max = 0, ball_mean = 0, page_max = 0;
     uint32_t ball_theta = 0;
     // warp search: per source its first pair and pair count; whether the last search
     // handed sources to the tile search (their pairs are then not in segments)
@@ -595,6 +601,11 @@ struct SearchArgs {
     uint32_t *brd_d;
     uint64_t brd_cap;
     unsigned long long *brd_count;
+    // source search by pages: the rows of eight arc slots (n_rows: the nodes' and the
+    // overflow rows'), pages, table buckets, queue entries and words of a group's map,
+    // groups resident on an SM
+    const uint4 *__restrict__ ell;
+    uint32_t n_rows, pg_cap, pg_buckets, pg_queue, pg_words, pg_resident;
 };
 
 // What a block needs to know about the tile it searches.
@@ -1270,6 +1281,655 @@ __global__ void __launch_bounds__(THREADS, (THREADS == NARROW ? CTAS_PER_SM : 1)
 }
 
 // ----------------------------------------------------------- source search ----
+// A group of W warps searches one source at a time (persistent: groups pop sources from
+// the work counter).  The bisection order puts a ball's nodes into runs of consecutive
+// internal ids: of the 32 nodes of a page (ids 32 p .. 32 p + 31) that a ball touches it
+// holds 17 to 24 on road-like graphs (balls of 500 to 3500 nodes), and four arcs of five
+// stay inside their page.  So the ball lives in shared memory as pages, not as hashed nodes:
+//   dist[32 s + i]   of node 32 pkey[s] + i:  2 d + 1 while the node is dirty (its distance
+//                    improved since its arcs were last relaxed), 2 d once it is clean,
+//                    PG_CLEAN while the search has not met it;
+//   table            page -> s: buckets of two entries (page << PG_BITS | s), the home bucket
+//                    at the page's low bits, read with one 8-byte load; a full bucket goes on
+//                    in the next.
+// One atomicMin on a node's word does all a relaxation needs: it lowers the distance, marks
+// the node dirty, and its old value says whether that improved it and whether the node
+// already sits in the near queue (it was dirty with a distance inside the bucket).
+//
+// Delta-stepping: a round takes the near queue's items, two lanes an item.  A lane loads
+// four of its item's eight arc slots (a row of eight slots per node, 64 bytes at 64 y, so
+// no CSR offset is read first; a node with more arcs goes on in a row of its own behind an
+// arc of weight 0), then issues the four table lookups, the four atomicMin and the pushes.
+// When the queue drains, a pass over the ball's pages takes the least pending distance and
+// collects the next bucket.  W = 1: four groups per block, lanes synchronise with
+// __syncwarp.  W > 1: one group per block, one barrier per round: a scan takes its item's
+// dirty bit with an atomicAnd, so scans and relaxations of a round need no barrier between
+// them (a distance improved before the scan is read by it; one improved after it makes the
+// node dirty again and pushes it).
+//
+// A source whose ball outgrows the pages stops and reports (source, bound, bucket end
+// reached, nodes met); the host searches it again with more pages or with the tile search.
+//
+// What bounds it is instruction issue and the latency of a round (one L2 trip for the rows,
+// then lookup and atomic in shared memory), not bandwidth: 1.07M-node join, 26.4M ball nodes
+// and 147M relaxed arcs in 1.2 ms, 0.91G warp instructions (6.2 an arc), 65% issue active.
+// Hashing every node instead (1.15G instructions, two probes chains and two atomics an arc,
+// CSR offsets before the arcs) took 1.48 ms there, 1.27 ms against 0.74 on the 264k-node join
+// and 2.32 against 1.09 with balls of 3,500 nodes (eight warps a ball).
+constexpr uint32_t PG_BITS = 11;  // a group's pages are numbered in 11 bits
+constexpr uint32_t PG_SLOT = (1u << PG_BITS) - 1;
+constexpr uint32_t PG_CLEAN = 0xFFFFFFFEu;
+constexpr uint32_t PG_NONE = 0xFFFFFFFFu;       // an empty table entry
+constexpr uint32_t PG_PAD = 0x80000001u;        // weight of an arc slot without an arc
+constexpr uint32_t PG_BOUND_MAX = 0x7FFFFFFEu;  // 2 d + 1 stays below PG_CLEAN
+constexpr uint32_t PG_ROW = 8;                  // arc slots per row
+constexpr uint64_t PG_ROWS_MAX = (uint64_t(1) << (32 - PG_BITS)) * 32 - 64;  // page ids fit beside the slot
+constexpr uint32_t PG_MAX = 1536;               // most pages of one group (196 KB of distances)
+__host__ __device__ constexpr int pg_groups(int W) { return W == 1 ? 4 : 1; }
+// control words of a group, behind its queues
+enum {
+    PC_PAGES, PC_CNT0, PC_CNT1, PC_CNT2, PC_MIN0, PC_MIN1, PC_FAIL, PC_ITEM, PC_BOUND, PC_BASE_LO, PC_BASE_HI, PC_FILL,
+    PC_STOP, PC_WORDS = 16
+};
+
+__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    return v;
+}
+
+// One warp: the first bin of the k-closest-pairs histogram where the cumulative count
+// reaches k, and the live bound lowered to that bin's upper edge.  Each lane sums its 64
+// consecutive bins (16 independent vector loads); the lane whose range holds the k-th
+// pair reads its bins again to find the bin.
+__device__ __forceinline__ void kcp_lower_bound(const SearchArgs &a, uint32_t lane) {
+    constexpr uint32_t PER = KCP_BINS / 32;
+    const uint4 *h4 = reinterpret_cast<const uint4 *>(a.kcp_hist) + lane * (PER / 4);
+    unsigned long long own = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < PER / 4; i++) {
+        const uint4 q = __ldcg(&h4[i]);
+        own += (unsigned long long)q.x + q.y + q.z + q.w;
+    }
+    unsigned long long incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= uint32_t(o)) incl += t;
+    }
+    const uint32_t reach = __ballot_sync(FULL, incl >= a.kcp_k);
+    if (reach && lane == uint32_t(__ffs(reach) - 1)) {
+        unsigned long long cum = incl - own;
+        uint32_t bin = lane * PER + PER - 1;
+        for (uint32_t i = 0; i < PER / 4; i++) {
+            const uint4 q = __ldcg(&h4[i]);
+            const uint32_t c4[4] = {q.x, q.y, q.z, q.w};
+            bool found = false;
+#pragma unroll
+            for (uint32_t j = 0; j < 4; j++) {
+                cum += c4[j];
+                if (!found && cum >= a.kcp_k) {
+                    bin = lane * PER + 4 * i + j;
+                    found = true;
+                }
+            }
+            if (found) break;
+        }
+        const unsigned long long edge = ((unsigned long long)(bin + 1) << a.hist_shift) - 1;
+        atomicMin(a.theta_live, uint32_t(min(edge, 0xFFFFFFFFull)));
+    }
+}
+
+template <int W>
+__device__ __forceinline__ void group_sync() {
+    if (W == 1) __syncwarp();
+    else __syncthreads();
+}
+
+// The slot of `page` (the same for every lane of the warp, which all call), inserting it if
+// absent; cap when the pages are used up.  Nothing leaves the table during a search, so an
+// empty entry in a bucket ends the probing.  W > 1: another warp may insert at the same time;
+// the entry is taken with a compare-and-swap, and a slot drawn for a page that another warp
+// inserted first is kept (spare) for the warp's next page.
+template <int W>
+__device__ __forceinline__ uint32_t page_slot(uint32_t *table, uint32_t *pkey, uint32_t *ctl, uint32_t page,
+                                              uint32_t bmask, uint32_t cap, uint32_t lane, uint32_t &spare) {
+    uint32_t b = page & bmask;
+    for (uint32_t probe = 0; probe < 4 * (bmask + 1); probe++) {
+        uint2 e = *reinterpret_cast<const uint2 *>(table + 2 * b);
+        if (W > 1) e = make_uint2(__shfl_sync(FULL, e.x, 0), __shfl_sync(FULL, e.y, 0));  // one view for all lanes
+        if ((e.x >> PG_BITS) == page) return e.x & PG_SLOT;
+        if ((e.y >> PG_BITS) == page) return e.y & PG_SLOT;
+        if (e.x != PG_NONE && e.y != PG_NONE) {
+            b = (b + 1) & bmask;
+            continue;
+        }
+        const uint32_t at = 2 * b + (e.x == PG_NONE ? 0u : 1u);
+        if (W == 1) {
+            const uint32_t s = ctl[PC_PAGES];
+            __syncwarp();
+            if (s >= cap) return cap;
+            if (lane == 0) {
+                table[at] = page << PG_BITS | s;
+                pkey[s] = page;
+                ctl[PC_PAGES] = s + 1;
+            }
+            __syncwarp();
+            return s;
+        }
+        uint32_t mine = spare;
+        if (mine == PG_NONE) {
+            if (lane == 0) mine = atomicAdd(&ctl[PC_PAGES], 1u);
+            mine = __shfl_sync(FULL, mine, 0);
+            if (mine >= cap) return cap;
+        }
+        uint32_t prev = 0;
+        if (lane == 0) {
+            pkey[mine] = page;
+            prev = atomicCAS(&table[at], PG_NONE, page << PG_BITS | mine);
+        }
+        prev = __shfl_sync(FULL, prev, 0);
+        spare = prev == PG_NONE ? PG_NONE : mine;
+        if (prev == PG_NONE) return mine;
+        if ((prev >> PG_BITS) == page) return prev & PG_SLOT;
+    }
+    return cap;
+}
+
+template <int W, bool HIER>
+__global__ void __launch_bounds__(32 * W * pg_groups(W), W == 1 ? 8 : 32 / W) k_source_search(SearchArgs a) {
+    constexpr uint32_t NT = 32 * W;
+    constexpr int G = pg_groups(W);
+    extern __shared__ __align__(16) uint32_t smem[];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t grp = W == 1 ? warp : 0, gw = W == 1 ? 0 : warp;  // group in the block, warp in the group
+    const uint32_t gt = gw * 32 + lane;
+    const uint32_t lt = (1u << lane) - 1;
+    const uint32_t cap = a.pg_cap, bmask = a.pg_buckets - 1, QS = a.pg_queue;
+    uint32_t *const dist = smem + grp * a.pg_words;
+    uint32_t *const table = dist + 32 * cap;
+    uint32_t *const pkey = table + 2 * a.pg_buckets;
+    uint32_t *const queues = pkey + cap;  // two near queues of QS 16-bit entries; emission keeps a hit mask per page
+    uint32_t *const ctl = queues + QS;
+    for (uint32_t i = gt; i < 8 * cap; i += NT)
+        reinterpret_cast<uint4 *>(dist)[i] = make_uint4(PG_CLEAN, PG_CLEAN, PG_CLEAN, PG_CLEAN);
+    for (uint32_t i = gt; i < a.pg_buckets / 2; i += NT)
+        reinterpret_cast<uint4 *>(table)[i] = make_uint4(PG_NONE, PG_NONE, PG_NONE, PG_NONE);
+    // telemetry: counted per source in registers, added to the group's totals when it ends
+    enum { W_SCANS, W_ARCS, W_SLOT_ARCS, W_ROUNDS, W_BOUNDS, W_SLOTS, W_PAGES, W_CYC_ROUND, W_CYC_BOUND, W_CYC_EMIT, W_N };
+    enum { M_BALL, M_SEG, M_PAGES, M_N };
+    __shared__ unsigned long long s_tel[G][W_N];
+    __shared__ uint32_t s_max[G][M_N];
+    __shared__ uint32_t s_wcnt[W];
+    if (gt < W_N) s_tel[grp][gt] = 0;
+    if (gt < M_N) s_max[grp][gt] = 0;
+    if (gt == 0) ctl[PC_STOP] = __ldcg(&a.ctl->err) != 0;
+    group_sync<W>();
+    if (ctl[PC_STOP]) return;
+    const uint32_t nR1 = a.nR_fixed ? a.nR_fixed : __ldcg(&a.ctl->r_count);
+    const uint32_t nitems = a.range_list ? a.ntiles : nR1;
+    const bool kcp = a.kcp_hist != nullptr;
+    uint32_t t_mark = uint32_t(clock());
+
+    for (;;) {
+        uint32_t item = 0;
+        if (W == 1) {
+            if (lane == 0) item = atomicAdd(&a.ctl->tile_next, 1u);
+            item = __shfl_sync(FULL, item, 0);
+        } else {
+            if (gt == 0) ctl[PC_ITEM] = atomicAdd(&a.ctl->tile_next, 1u);
+            __syncthreads();
+            item = ctl[PC_ITEM];
+        }
+        if (item >= nitems) break;
+        const uint32_t si = a.range_list ? a.range_list[item].x : item;
+        bool skip = si >= nR1;  // never past R
+        const uint32_t y0 = skip ? 0u : a.src[si];
+        if (!skip && y0 >= a.n_nodes) {  // (the same for every thread of the group)
+            if (gt == 0) record_check(a.ctl, 11, si, y0);
+            skip = true;
+        }
+        if (skip) {
+            group_sync<W>();  // every thread has read the item
+            continue;
+        }
+        uint32_t bound = a.bound;
+        const uint32_t *sbits = a.sbits;
+        unsigned long long prefix = 0;
+        uint32_t inst = 0;
+        if (a.inst_first) {
+            // the query whose sources hold si: the last with inst_first <= si
+            uint32_t lo = 0, hi = a.inst_count - 1;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi + 1) >> 1;
+                if (a.inst_first[mid] <= si) lo = mid;
+                else hi = mid - 1;
+            }
+            inst = lo;
+            bound = a.inst_bound[lo];
+            sbits = a.inst_sbits[lo];
+            prefix = (unsigned long long)lo << a.inst_shift;
+        }
+        uint32_t delta = a.delta;
+        if (a.tile_bound) {  // a batch: the source's instance, its bound and bucket width
+            inst = a.tile_inst[si];
+            bound = a.tile_bound[si];
+            delta = a.tile_delta[si];
+        }
+        // (the host runs this search only where no distance within the bound passes
+        // PG_BOUND_MAX, so the cut changes nothing)
+        bound = min(bound, PG_BOUND_MAX);
+        delta = min(delta, 0x80000000u);
+        const bool swap = a.inst_swap ? a.inst_swap[inst] != 0 : a.swap_uv != 0;
+        const unsigned long long u = __ldg(&a.iperm[y0]);
+        const uint32_t t_source = uint32_t(clock());
+        uint32_t part_lo = 0, part_hi = 0xFFFFFFFFu;  // the hierarchical variant: the source's part
+        if (HIER) {
+            const uint2 r = a.src_range[si];
+            part_lo = r.x;
+            part_hi = r.y;
+        }
+        // the source, at distance 0, is the only item of the near queue
+        if (gt == 0) {
+            const uint32_t page = y0 >> 5;
+            table[2 * (page & bmask)] = page << PG_BITS;
+            pkey[0] = page;
+            dist[y0 & 31] = 1;
+            reinterpret_cast<uint16_t *>(queues)[0] = uint16_t(y0 & 31);
+            ctl[PC_PAGES] = 1;
+            if (W > 1) {
+                ctl[PC_CNT0] = ctl[PC_CNT0 + 1] = ctl[PC_CNT0 + 2] = 0;
+                ctl[PC_MIN0] = ctl[PC_MIN0 + 1] = PG_NONE;
+                ctl[PC_FAIL] = 0;
+                // k closest pairs: the live k-th distance bound (Algorithm 3's global threshold)
+                // caps the source's bound, and is read again at every bucket boundary
+                if (kcp) ctl[PC_BOUND] = min(bound, __ldcg(a.theta_live));
+            }
+        }
+        group_sync<W>();
+        if (kcp) bound = W == 1 ? min(bound, __ldcg(a.theta_live)) : ctl[PC_BOUND];
+        uint16_t *qcur = reinterpret_cast<uint16_t *>(queues), *qnext = qcur + QS;
+        uint32_t ncur = 1, rot = 0;  // W > 1: the next round's count is ctl[PC_CNT0 + (rot + 1) % 3]
+        uint32_t n_scans = 0, n_arcs = 0, n_rounds = 0, n_bounds = 0, cyc_round = 0, cyc_bound = 0;
+        uint32_t spare = PG_NONE;
+        bool fail = false;
+        uint32_t tau = min(delta, bound + 1);  // end of the bucket
+
+        for (;;) {
+            // ---- rounds of the current bucket
+            while (ncur && !fail) {
+                n_rounds++;
+                uint32_t nnext = 0;
+                const uint32_t rot1 = rot == 2 ? 0 : rot + 1, rot2 = rot1 == 2 ? 0 : rot1 + 1;
+                if (W > 1 && gt == 0) ctl[PC_CNT0 + rot2] = 0;
+                const uint32_t tau2 = 2 * tau;  // <= 2 (bound + 1) < 2^32
+                for (uint32_t c0 = 16 * gw; c0 < ncur && !fail; c0 += 16 * W) {
+                    // two lanes an item: lane 2 i + h takes arc slots 4 h .. 4 h + 3 of item c0 + i
+                    const uint32_t j = c0 + (lane >> 1);
+                    uint4 r0 = make_uint4(0, PG_PAD, 0, PG_PAD), r1 = r0;
+                    uint32_t word = 0;
+                    if (j < ncur) {
+                        const uint32_t x = qcur[j];
+                        if (!RN_BAD(x < 32 * cap, 12, j, x)) {
+                            const uint32_t y = pkey[x >> 5] * 32 + (x & 31);
+                            if (!RN_BAD(y < a.n_rows, 13, x, y)) {
+                                const uint4 *row = a.ell + size_t(y) * (PG_ROW / 2) + (lane & 1) * 2;
+                                r0 = __ldg(row);
+                                r1 = __ldg(row + 1);
+                            }
+                            if (W == 1) {
+                                word = dist[x];  // (cleared by one lane: the other may read it before or after)
+                                if (!(lane & 1)) dist[x] = word & ~1u;
+                            } else if (!(lane & 1)) {
+                                word = atomicAnd(&dist[x], ~1u);
+                            }
+                        }
+                    }
+                    if (W == 1) __syncwarp();  // the scans' stores before any relaxation
+                    else word = __shfl_sync(FULL, word, lane & 30);
+                    const uint32_t d = word >> 1;
+                    n_scans += min(16u, ncur - c0);
+                    n_arcs += 4 - (r0.y >> 31) - (r0.w >> 31) - (r1.y >> 31) - (r1.w >> 31);
+                    const uint32_t y[4] = {r0.x, r0.z, r1.x, r1.z};
+                    uint32_t nd[4] = {d + r0.y, d + r0.w, d + r1.y, d + r1.w};  // a pad's is above any bound
+                    uint32_t s[4];
+                    bool miss[4];
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        // (a part's overflow rows lie past the nodes and lead back into the part)
+                        if (HIER && (y[k] < part_lo || y[k] >= part_hi) && y[k] < a.n_nodes) nd[k] = INF;
+                        if (nd[k] <= bound && RN_BAD(y[k] < a.n_rows, 16, c0 + lane, y[k])) nd[k] = INF;
+                        const uint32_t page = y[k] >> 5;
+                        const uint2 e = *reinterpret_cast<const uint2 *>(table + 2 * (page & bmask));
+                        s[k] = (e.x >> PG_BITS) == page ? e.x : e.y;
+                        miss[k] = nd[k] <= bound && (s[k] >> PG_BITS) != page;
+                    }
+                    // pages the table's home bucket does not hold (mostly pages met for the
+                    // first time), one distinct page after another
+                    uint32_t need;
+                    while ((need = __ballot_sync(FULL, miss[0] || miss[1] || miss[2] || miss[3])) != 0) {
+                        const uint32_t own = miss[0] ? y[0] : miss[1] ? y[1] : miss[2] ? y[2] : y[3];
+                        const uint32_t page = __shfl_sync(FULL, own, __ffs(need) - 1) >> 5;
+                        const uint32_t slot = page_slot<W>(table, pkey, ctl, page, bmask, cap, lane, spare);
+                        if (slot >= cap) fail = true;
+#pragma unroll
+                        for (int k = 0; k < 4; k++)
+                            if (miss[k] && (y[k] >> 5) == page) {
+                                s[k] = slot;
+                                miss[k] = false;
+                                if (slot >= cap) nd[k] = INF;
+                            }
+                    }
+                    uint32_t old[4];
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        s[k] = (s[k] & PG_SLOT) * 32 + (y[k] & 31);
+                        old[k] = nd[k] <= bound ? atomicMin(&dist[s[k]], 2 * nd[k] + 1) : 0u;
+                    }
+                    // a node improved inside the bucket joins the near queue, unless it is in it
+                    // already (it was dirty with a distance inside the bucket)
+                    bool push[4];
+                    uint32_t pb[4], at = nnext;
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        const uint32_t nw = 2 * nd[k] + 1;
+                        push[k] = nw < old[k] && nw < tau2 && (!(old[k] & 1) || old[k] > tau2);
+                        pb[k] = __ballot_sync(FULL, push[k]);
+                        nnext += __popc(pb[k]);
+                    }
+                    if (W > 1) {
+                        const uint32_t cnt = nnext;
+                        nnext = 0;
+                        if (cnt) {
+                            if (lane == 0) at = atomicAdd(&ctl[PC_CNT0 + rot1], cnt);
+                            at = __shfl_sync(FULL, at, 0);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        const uint32_t qi = at + __popc(pb[k] & lt);
+                        if (push[k] && qi < QS) qnext[qi] = uint16_t(s[k]);  // (a full queue leaves it dirty)
+                        at += __popc(pb[k]);
+                    }
+                }
+                if (W == 1) {
+                    __syncwarp();
+                } else {
+                    if (fail && lane == 0) ctl[PC_FAIL] = 1;
+                    __syncthreads();
+                    nnext = ctl[PC_CNT0 + rot1];
+                    fail = ctl[PC_FAIL] != 0;
+                    rot = rot1;
+                }
+                ncur = min(nnext, QS);
+                uint16_t *t = qcur;
+                qcur = qnext;
+                qnext = t;
+            }
+            {
+                const uint32_t t = uint32_t(clock());
+                cyc_round += t - t_mark;
+                t_mark = t;
+            }
+            if (fail) break;
+            // ---- the near queue is empty: the next bucket
+            if (kcp) {
+                if (W == 1) {
+                    bound = min(bound, __ldcg(a.theta_live));  // the same for every lane
+                } else {
+                    __syncthreads();
+                    if (gt == 0) ctl[PC_BOUND] = min(bound, __ldcg(a.theta_live));
+                    __syncthreads();
+                    bound = ctl[PC_BOUND];
+                }
+            }
+            const uint32_t pages = min(ctl[PC_PAGES], cap);
+            const uint32_t rot1 = rot == 2 ? 0 : rot + 1, rot2 = rot1 == 2 ? 0 : rot1 + 1;
+            const uint32_t mslot = PC_MIN0 + (n_bounds & 1);
+            n_bounds++;
+            if (W > 1 && gt == 0) {
+                ctl[PC_CNT0 + rot2] = 0;
+                ctl[PC_MIN0 + (n_bounds & 1)] = PG_NONE;  // (the next boundary's: a round's barrier away)
+            }
+            // least distance of the dirty nodes; those below lim go to the near queue (as many
+            // as fit: the rest stay dirty for the next pass)
+            uint32_t nq = 0;
+            auto collect = [&](uint32_t lim) {
+                uint32_t m = PG_NONE;
+#pragma unroll 4
+                for (uint32_t p = gw; p < pages; p += W) {
+                    const uint32_t w = dist[32 * p + lane];
+                    const uint32_t d = (w & 1) ? w >> 1 : PG_NONE;
+                    m = min(m, d);
+                    const bool take = d < lim;
+                    const uint32_t b = __ballot_sync(FULL, take);
+                    uint32_t at = nq;
+                    if (W > 1 && b) {
+                        if (lane == 0) at = atomicAdd(&ctl[PC_CNT0 + rot1], uint32_t(__popc(b)));
+                        at = __shfl_sync(FULL, at, 0);
+                    }
+                    const uint32_t qi = at + __popc(b & lt);
+                    if (take && qi < QS) qcur[qi] = uint16_t(32 * p + lane);
+                    if (W == 1) nq += __popc(b);
+                }
+                return __reduce_min_sync(FULL, m);
+            };
+            const uint32_t top = bound + 1;
+            uint32_t lim = tau < top && top - tau > delta ? tau + delta : top;
+            uint32_t m = collect(lim);
+            if (W > 1) {
+                if (lane == 0) atomicMin(&ctl[mslot], m);
+                __syncthreads();
+                m = ctl[mslot];
+            }
+            // nothing pending within the bound: the search is complete (a bound lowered by k
+            // closest pairs leaves dirty nodes above it, which are never taken)
+            if (m > bound) break;
+            if (m >= lim) {
+                // no pending node in the next bucket: skip to the one holding m
+                const unsigned long long t = ((unsigned long long)(m / delta) + 1) * delta;
+                lim = t < top ? uint32_t(t) : top;
+                nq = 0;
+                collect(lim);
+                if (W > 1) __syncthreads();
+            }
+            tau = lim;
+            if (W > 1) {
+                nq = ctl[PC_CNT0 + rot1];
+                rot = rot1;
+            }
+            ncur = min(nq, QS);
+            if (W == 1) __syncwarp();
+            {
+                const uint32_t t = uint32_t(clock());
+                cyc_bound += t - t_mark;
+                t_mark = t;
+            }
+        }
+
+        // ---- emission: the pairs of the ball's S nodes, page by page (warp gw takes pages gw,
+        // gw + W, ...): a page's 32 membership bits are one word of the S bitmap.  First the
+        // hits of every page (kept as masks where the queues were), then their range of the
+        // output, then the pairs.
+        group_sync<W>();
+        const uint32_t pages = min(ctl[PC_PAGES], cap);
+        uint32_t fill = 0, cnt = 0, slot_arcs = 0;
+        for (uint32_t p0 = gw; p0 < pages; p0 += 32 * W) {
+            const uint32_t pl = p0 + lane * W;
+            const uint32_t key = pl < pages ? pkey[pl] : PG_NONE;
+            const bool real = pl < pages && 32ull * key < a.n_nodes;  // (the last words' spare bits are zero)
+            const uint32_t sw = real && !fail ? __ldg(&sbits[key]) : 0u;
+            uint32_t bw = 0;
+            if (HIER) bw = real && !fail ? __ldg(&a.border_bits[key]) : 0u;
+            uint32_t hits = 0;
+            const uint32_t np = min(32u, (pages - p0 + W - 1) / W);
+#pragma unroll 4
+            for (uint32_t i = 0; i < np; i++) {
+                const uint32_t w = dist[32 * (p0 + i * W) + lane];
+                const uint32_t yy = __shfl_sync(FULL, key, i) * 32 + lane, swi = __shfl_sync(FULL, sw, i);
+                const bool met = w < PG_CLEAN;
+                fill += __popc(__ballot_sync(FULL, met));
+                if (met && yy < a.n_nodes) slot_arcs += __ldg(&a.row_ptr[yy + 1]) - __ldg(&a.row_ptr[yy]);
+                const bool in = met && (w >> 1) <= bound && ((swi >> lane) & 1u);
+                const uint32_t mask = __ballot_sync(FULL, in);
+                cnt += __popc(mask);
+                if (lane == i) hits = mask;
+                if (HIER) {
+                    // the routes to the part's border nodes (the inside routes that the search
+                    // from an exit arc's far end continues)
+                    const uint32_t bwi = __shfl_sync(FULL, bw, i);
+                    const bool brd = met && ((bwi >> lane) & 1u);
+                    const uint32_t bb = __ballot_sync(FULL, brd);
+                    if (bb) {
+                        unsigned long long at = 0;
+                        if (lane == 0) at = atomicAdd(a.brd_count, (unsigned long long)__popc(bb));
+                        at = __shfl_sync(FULL, at, 0) + __popc(bb & lt);
+                        if (brd && at < a.brd_cap) {
+                            a.brd_key[at] = ((unsigned long long)si << 32) | yy;
+                            a.brd_d[at] = w >> 1;
+                        }
+                    }
+                }
+            }
+            if (pl < pages) queues[pl] = hits;
+        }
+        uint32_t before = 0, total = cnt, ball = fill;
+        unsigned long long base = 0;
+        if (W > 1) {
+            if (lane == 0) {
+                s_wcnt[warp] = cnt;
+                if (warp == 0) ctl[PC_FILL] = 0;
+            }
+            __syncthreads();
+            if (lane == 0) atomicAdd(&ctl[PC_FILL], fill);
+            total = 0;
+#pragma unroll
+            for (int w = 0; w < W; w++) {
+                if (w < int(warp)) before += s_wcnt[w];
+                total += s_wcnt[w];
+            }
+        }
+        if (!fail) {
+            if (gt == 0) {
+                if (total) {
+                    base = atomicAdd(&a.ctl->pairs, (unsigned long long)total);
+                    if (a.inst_pairs) atomicAdd(&a.inst_pairs[inst], (unsigned long long)total);
+                }
+                if (a.seg) a.seg[si] = make_uint2(uint32_t(base), total);
+                if (W > 1) {
+                    ctl[PC_BASE_LO] = uint32_t(base);
+                    ctl[PC_BASE_HI] = uint32_t(base >> 32);
+                }
+            }
+        }
+        if (W == 1) {
+            base = __shfl_sync(FULL, base, 0);
+            __syncwarp();
+        } else {
+            __syncthreads();
+            base = (unsigned long long)ctl[PC_BASE_HI] << 32 | ctl[PC_BASE_LO];
+            ball = ctl[PC_FILL];
+        }
+        if (!fail) {
+            unsigned long long pos = base + before;
+#pragma unroll 4
+            for (uint32_t p = gw; p < pages; p += W) {
+                const uint32_t mask = queues[p];
+                if ((mask >> lane) & 1u) {
+                    const uint32_t yy = pkey[p] * 32 + lane, dd = dist[32 * p + lane] >> 1;
+                    const unsigned long long idx = pos + __popc(mask & lt);
+                    const uint32_t v = __ldg(&a.iperm[yy]);
+                    if (idx < a.out_cap) {
+                        a.out_key[idx] = prefix | (swap ? ((unsigned long long)v << a.vbits) | u
+                                                        : (u << a.vbits) | (unsigned long long)v);
+                        a.out_d[idx] = dd;
+                    }
+                    if (kcp) atomicAdd(&a.kcp_hist[dd >> a.hist_shift], 1u);
+                }
+                pos += __popc(mask);
+            }
+            if (kcp && total && gw == 0) {
+                // the source's pairs are counted: once k pairs exist, lower the live bound
+                // to the edge of the first histogram bin where the pairs emitted so far
+                // reach k (exact, distinct pairs: the k-th distance cannot lie above it).
+                // The group whose pairs reach k does it, then the group whose pairs cross
+                // each further multiple of k/64 (not every source: each lowering reads the
+                // whole histogram)
+                const unsigned long long emitted = base + total;
+                const unsigned long long step = a.kcp_k / 64 + 1;
+                if (emitted >= a.kcp_k && (base < a.kcp_k || base / step != emitted / step)) kcp_lower_bound(a, lane);
+            }
+        }
+        n_arcs = __reduce_add_sync(FULL, n_arcs);
+        slot_arcs = __reduce_add_sync(FULL, slot_arcs);
+        group_sync<W>();  // the pages are read before they are cleared
+        for (uint32_t i = gt; i < 8 * pages; i += NT)
+            reinterpret_cast<uint4 *>(dist)[i] = make_uint4(PG_CLEAN, PG_CLEAN, PG_CLEAN, PG_CLEAN);
+        for (uint32_t i = gt; i < a.pg_buckets / 2; i += NT)
+            reinterpret_cast<uint4 *>(table)[i] = make_uint4(PG_NONE, PG_NONE, PG_NONE, PG_NONE);
+        const uint32_t t_end = uint32_t(clock());
+        unsigned long long *const tel = s_tel[grp];
+        if (lane == 0) {
+            if (W == 1) {
+                tel[W_SCANS] += n_scans;
+                tel[W_ARCS] += n_arcs;
+                if (!fail) tel[W_SLOT_ARCS] += slot_arcs;
+            } else {
+                atomicAdd(&tel[W_SCANS], (unsigned long long)n_scans);
+                atomicAdd(&tel[W_ARCS], (unsigned long long)n_arcs);
+                if (!fail) atomicAdd(&tel[W_SLOT_ARCS], (unsigned long long)slot_arcs);
+            }
+        }
+        if (gt == 0) {
+            if (!fail) {
+                tel[W_SLOTS] += ball;
+                tel[W_PAGES] += pages;
+                s_max[grp][M_BALL] = max(s_max[grp][M_BALL], ball);
+                s_max[grp][M_SEG] = max(s_max[grp][M_SEG], total);
+                s_max[grp][M_PAGES] = max(s_max[grp][M_PAGES], pages);
+                if (a.inst_ball) atomicMax(&a.inst_ball[inst], pages);
+            } else {
+                a.failed[atomicAdd(&a.ctl->n_failed, 1u)] = make_uint4(si, bound, tau, max(ball, 1u));
+            }
+            tel[W_ROUNDS] += n_rounds;
+            tel[W_BOUNDS] += n_bounds;
+            tel[W_CYC_ROUND] += cyc_round;
+            tel[W_CYC_BOUND] += cyc_bound;
+            tel[W_CYC_EMIT] += t_end - t_mark;
+            // a batch: the instance's SM cycles, this group holding its share of the SM
+            if (a.inst_cycles) atomicAdd(&a.inst_cycles[inst], (unsigned long long)(t_end - t_source) / a.pg_resident);
+        }
+        t_mark = t_end;
+        group_sync<W>();
+    }
+    group_sync<W>();
+    if (gt == 0) {
+        const unsigned long long *tel = s_tel[grp];
+        atomicAdd(&a.ctl->scans, tel[W_SCANS]);
+        atomicAdd(&a.ctl->dirty_groups, tel[W_SCANS]);
+        atomicAdd(&a.ctl->round_items, tel[W_SCANS]);
+        atomicAdd(&a.ctl->round_arcs, tel[W_ARCS]);
+        atomicAdd(&a.ctl->slot_arcs, tel[W_SLOT_ARCS]);
+        atomicAdd(&a.ctl->slots, tel[W_SLOTS]);
+        atomicAdd(&a.ctl->slot_lanes, tel[W_SLOTS]);
+        atomicAdd(&a.ctl->pages, tel[W_PAGES]);
+        atomicAdd(&a.ctl->rounds, tel[W_ROUNDS]);
+        atomicAdd(&a.ctl->boundaries, tel[W_BOUNDS]);
+        atomicAdd(&a.ctl->cyc_round, tel[W_CYC_ROUND]);
+        atomicAdd(&a.ctl->cyc_bound, tel[W_CYC_BOUND]);
+        atomicAdd(&a.ctl->cyc_emit, tel[W_CYC_EMIT]);
+        atomicMax(&a.ctl->max_fill, s_max[grp][M_BALL]);
+        atomicMax(&a.ctl->src_max_ball, s_max[grp][M_BALL]);
+        atomicMax(&a.ctl->src_max_pages, s_max[grp][M_PAGES]);
+        atomicMax(&a.ctl->max_seg, s_max[grp][M_SEG]);
+    }
+}
+
+// ----------------------------------------------------- hashed source search ----
+// The search of graphs whose node ids carry no locality (loaded without the bisection
+// order, or with hubs), where a page would hold a node or two: the ball's nodes are hashed
+// one by one.
+//
 // One warp searches one source at a time (persistent: warps pop sources from the work
 // counter).  The source's ball lives in a map of MS slots in shared memory that only this
 // warp touches:
@@ -1334,56 +1994,8 @@ __device__ __forceinline__ uint32_t src_slot(uint32_t *key, uint32_t y, uint32_t
     return EMPTY;
 }
 
-__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    return v;
-}
-
-// One warp: the first bin of the k-closest-pairs histogram where the cumulative count
-// reaches k, and the live bound lowered to that bin's upper edge.  Each lane sums its 64
-// consecutive bins (16 independent vector loads); the lane whose range holds the k-th
-// pair reads its bins again to find the bin.
-__device__ __forceinline__ void kcp_lower_bound(const SearchArgs &a, uint32_t lane) {
-    constexpr uint32_t PER = KCP_BINS / 32;
-    const uint4 *h4 = reinterpret_cast<const uint4 *>(a.kcp_hist) + lane * (PER / 4);
-    unsigned long long own = 0;
-#pragma unroll
-    for (uint32_t i = 0; i < PER / 4; i++) {
-        const uint4 q = __ldcg(&h4[i]);
-        own += (unsigned long long)q.x + q.y + q.z + q.w;
-    }
-    unsigned long long incl = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long t = __shfl_up_sync(FULL, incl, o);
-        if (lane >= uint32_t(o)) incl += t;
-    }
-    const uint32_t reach = __ballot_sync(FULL, incl >= a.kcp_k);
-    if (reach && lane == uint32_t(__ffs(reach) - 1)) {
-        unsigned long long cum = incl - own;
-        uint32_t bin = lane * PER + PER - 1;
-        for (uint32_t i = 0; i < PER / 4; i++) {
-            const uint4 q = __ldcg(&h4[i]);
-            const uint32_t c4[4] = {q.x, q.y, q.z, q.w};
-            bool found = false;
-#pragma unroll
-            for (uint32_t j = 0; j < 4; j++) {
-                cum += c4[j];
-                if (!found && cum >= a.kcp_k) {
-                    bin = lane * PER + 4 * i + j;
-                    found = true;
-                }
-            }
-            if (found) break;
-        }
-        const unsigned long long edge = ((unsigned long long)(bin + 1) << a.hist_shift) - 1;
-        atomicMin(a.theta_live, uint32_t(min(edge, 0xFFFFFFFFull)));
-    }
-}
-
 template <uint32_t MS, bool HIER>
-__global__ void __launch_bounds__(src_warps(MS) * 32, SRC_BLOCKS_PER_SM) k_source_search(SearchArgs a) {
+__global__ void __launch_bounds__(src_warps(MS) * 32, SRC_BLOCKS_PER_SM) k_hash_search(SearchArgs a) {
     constexpr uint32_t QS = src_qcap(MS);
     constexpr int AP = 4;  // arcs per lane in flight
     extern __shared__ __align__(16) uint32_t smem[];  // (sixteen-byte stores clear the maps)
@@ -1840,7 +2452,7 @@ __global__ void __launch_bounds__(src_warps(MS) * 32, SRC_BLOCKS_PER_SM) k_sourc
 // bucket boundaries split the map between the warps.  The protocol and the results
 // are the warp search's.
 template <uint32_t MS, uint32_t W>
-__global__ void __launch_bounds__(W * 32, (3 * 8192) / MS) k_source_coop(SearchArgs a) {
+__global__ void __launch_bounds__(W * 32, (3 * 8192) / MS) k_hash_coop(SearchArgs a) {
     constexpr uint32_t QS = src_qcap(MS);
     constexpr uint32_t NT = W * 32;
     constexpr int AP = 4;
@@ -2910,10 +3522,10 @@ static void launch_source(const SearchArgs &a, uint32_t grid, cudaStream_t st) {
     constexpr uint32_t smem = src_warps(MS) * src_words(MS) * 4;
     static std::once_flag once[MAX_DEVICES];
     std::call_once(once[attr_device()], [&] {
-        RN_CUDA(cudaFuncSetAttribute(k_source_search<MS, HIER>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-        RN_CUDA(cudaFuncSetAttribute(k_source_search<MS, HIER>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        RN_CUDA(cudaFuncSetAttribute(k_hash_search<MS, HIER>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+        RN_CUDA(cudaFuncSetAttribute(k_hash_search<MS, HIER>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     });
-    k_source_search<MS, HIER><<<grid, src_warps(MS) * 32, smem, st>>>(a);
+    k_hash_search<MS, HIER><<<grid, src_warps(MS) * 32, smem, st>>>(a);
     RN_CUDA(cudaGetLastError());
 }
 
@@ -2928,17 +3540,17 @@ static void launch_coop(const SearchArgs &a, uint32_t grid, cudaStream_t st) {
     constexpr uint32_t W = coop_warps(MS), smem = src_words(MS) * 4;
     static std::once_flag once[MAX_DEVICES];
     std::call_once(once[attr_device()], [&] {
-        RN_CUDA(cudaFuncSetAttribute(k_source_coop<MS, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-        RN_CUDA(cudaFuncSetAttribute(k_source_coop<MS, W>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        RN_CUDA(cudaFuncSetAttribute(k_hash_coop<MS, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+        RN_CUDA(cudaFuncSetAttribute(k_hash_coop<MS, W>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     });
-    k_source_coop<MS, W><<<grid, W * 32, smem, st>>>(a);
+    k_hash_coop<MS, W><<<grid, W * 32, smem, st>>>(a);
     RN_CUDA(cudaGetLastError());
 }
 
 template <uint32_t MS>
 static int source_occupancy() {
     int b = 0;
-    RN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_source_search<MS, false>, src_warps(MS) * 32,
+    RN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_hash_search<MS, false>, src_warps(MS) * 32,
                                                           src_warps(MS) * src_words(MS) * 4));
     return b;
 }
@@ -2951,7 +3563,7 @@ static int coop_occupancy() {
         return source_occupancy<MS>();
     } else {
         int b = 0;
-        RN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_source_coop<MS, coop_warps(MS)>, coop_warps(MS) * 32,
+        RN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_hash_coop<MS, coop_warps(MS)>, coop_warps(MS) * 32,
                                                               src_words(MS) * 4));
         return b;
     }
@@ -2975,12 +3587,209 @@ static uint32_t *ensure_slist(Workspace *ws) {
     return ws->slist;
 }
 
+// ---- the search by pages: rows and launch shapes
+
+// Rows of eight arc slots from the CSR arrays; the slots past a node's arcs are pads.
+__global__ void k_rows(const uint32_t *__restrict__ row_ptr, const uint2 *__restrict__ adj, uint32_t n, uint2 *rows) {
+    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < uint64_t(n) * PG_ROW;
+         i += uint64_t(gridDim.x) * blockDim.x) {
+        const uint32_t y = uint32_t(i / PG_ROW), k = uint32_t(i % PG_ROW);
+        const uint32_t b = row_ptr[y], deg = row_ptr[y + 1] - b;
+        rows[i] = k < deg && (deg <= PG_ROW || k + 1 < PG_ROW) ? adj[b + k] : make_uint2(y, PG_PAD);
+    }
+}
+
+// The nodes of more than eight arcs: the eighth slot an arc of weight 0 to the node's first
+// overflow row (heavy[i] = node, row), which holds the next arcs, and so on.
+__global__ void k_rows_heavy(const uint32_t *__restrict__ row_ptr, const uint2 *__restrict__ adj,
+                             const uint2 *__restrict__ heavy, uint32_t count, uint2 *rows) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+        uint32_t row = heavy[i].x, next = heavy[i].y, at = row_ptr[row] + PG_ROW - 1;
+        uint32_t left = row_ptr[row + 1] - at;
+        for (;;) {
+            rows[size_t(row) * PG_ROW + PG_ROW - 1] = make_uint2(next, 0);
+            row = next++;
+            const uint32_t here = left <= PG_ROW ? left : PG_ROW - 1;
+            for (uint32_t k = 0; k < PG_ROW; k++)
+                rows[size_t(row) * PG_ROW + k] = k < here ? adj[at + k] : make_uint2(row, PG_PAD);
+            at += here;
+            left -= here;
+            if (!left) break;
+        }
+    }
+}
+
+// A graph's rows at node ids shifted by node_off, its overflow rows at row virt_at on.
+__global__ void k_rows_copy(const uint2 *__restrict__ in, uint32_t n, uint32_t nvirt, uint32_t node_off, uint32_t virt_at,
+                            uint2 *out) {
+    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < (uint64_t(n) + nvirt) * PG_ROW;
+         i += uint64_t(gridDim.x) * blockDim.x) {
+        const uint32_t y = uint32_t(i / PG_ROW), k = uint32_t(i % PG_ROW);
+        uint2 e = in[i];
+        e.x = e.x < n ? e.x + node_off : virt_at + (e.x - n);
+        out[size_t(y < n ? y + node_off : virt_at + (y - n)) * PG_ROW + k] = e;
+    }
+}
+
+static uint32_t rows_grid(uint64_t slots) { return uint32_t(std::max<uint64_t>(1, std::min<uint64_t>((slots + 255) / 256, 16384))); }
+
+static void rows_copy(const DeviceGraph &g, uint32_t node_off, uint32_t virt_at, uint4 *out, cudaStream_t st) {
+    const uint64_t slots = (uint64_t(g.n) + g.nvirt) * PG_ROW;
+    if (!slots) return;
+    k_rows_copy<<<rows_grid(slots), 256, 0, st>>>(reinterpret_cast<const uint2 *>(g.ell), g.n, g.nvirt, node_off, virt_at,
+                                                  reinterpret_cast<uint2 *>(out));
+    RN_CUDA(cudaGetLastError());
+}
+
+// Whether the graph is searched by pages, and its rows.  The pages pay where a ball fills
+// them: two arcs of five or more stay inside a page (a road network in bisection order: four
+// of five; random ids: none).  A hub would put its arcs into a long chain of overflow rows,
+// one round each, so graphs with nodes of more than 64 arcs keep the hashed search.
+static void build_rows(const HostGraph &g, DeviceGraph *d) {
+    uint64_t inside = 0, nvirt = 0;
+    uint32_t max_deg = 0, max_w = 0;
+    std::vector<uint2> heavy;
+    for (uint32_t y = 0; y < g.n; y++) {
+        const uint32_t deg = g.row_ptr[y + 1] - g.row_ptr[y];
+        max_deg = std::max(max_deg, deg);
+        for (uint32_t e = g.row_ptr[y]; e < g.row_ptr[y + 1]; e++) {
+            inside += (g.col[e] >> 5) == (y >> 5);
+            max_w = std::max(max_w, g.w[e]);
+        }
+        if (deg > PG_ROW) {
+            heavy.push_back(make_uint2(y, uint32_t(g.n + nvirt)));
+            // the first row holds 7 arcs, each overflow row 7 more, the last one 8
+            nvirt += (deg - PG_ROW + PG_ROW - 2) / (PG_ROW - 1);
+        }
+    }
+    d->far = g.n ? uint64_t(g.n - 1) * max_w : 0;
+    d->paged = max_deg <= 64 && 5 * inside >= 2 * g.arcs() && g.n + nvirt <= PG_ROWS_MAX;
+    if (!d->paged) return;
+    d->nvirt = uint32_t(nvirt);
+    d->row_chain = max_deg <= PG_ROW ? 0 : (max_deg - PG_ROW + PG_ROW - 2) / (PG_ROW - 1);
+    d->ell = (uint4 *)device_alloc(std::max<uint64_t>(g.n + nvirt, 1) * PG_ROW * 8);
+    uint2 *rows = reinterpret_cast<uint2 *>(d->ell);
+    const uint2 *adj = reinterpret_cast<const uint2 *>(d->adj);
+    if (g.n) k_rows<<<rows_grid(uint64_t(g.n) * PG_ROW), 256>>>(d->row_ptr, adj, g.n, rows);
+    RN_CUDA(cudaGetLastError());
+    uint2 *dh = nullptr;
+    if (!heavy.empty()) {
+        dh = (uint2 *)device_alloc(heavy.size() * 8);
+        const cudaError_t e = cudaMemcpy(dh, heavy.data(), heavy.size() * 8, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) {
+            const uint32_t count = uint32_t(heavy.size());
+            k_rows_heavy<<<std::min<uint32_t>((count + 255) / 256, 4096), 256>>>(d->row_ptr, adj, dh, count, rows);
+        }
+    }
+    const cudaError_t e = cudaDeviceSynchronize();
+    device_free(dh);
+    RN_CUDA(e);
+    RN_CUDA(cudaGetLastError());
+}
+
+// Balls up to this size go to the source search by default; past it the tile search shares
+// the work of a tile's sources.
+constexpr double PG_BALL_MAX = 20000.0;
+
+// Whether a query with bound theta is searched by pages (a distance is held in 31 bits).
+static bool by_pages(const DeviceGraph &g, uint32_t theta) {
+    return g.paged && (theta <= PG_BOUND_MAX || g.far <= PG_BOUND_MAX);
+}
+
+// A map of about p pages: never more than the graph or a group's shared memory holds.
+static uint32_t page_cap(const DeviceGraph &g, double p) {
+    const double all = double((uint64_t(g.n) + g.nvirt + 31) / 32 + 33);  // (and a spare page per warp)
+    const uint32_t c = uint32_t(std::min({std::max(p, 8.0), all, double(PG_MAX)}));
+    return std::min<uint32_t>((std::max<uint32_t>(c, 8) + 3) / 4 * 4, PG_MAX);
+}
+
+// Page counts of maps taken from an estimate or a measured ball, so that few launches serve
+// many sources: a fifth to a third apart.  PG_MAX + 1 when even the largest is too small.
+static uint32_t page_class(double pages) {
+    for (uint32_t c : {16u, 24u, 32u, 40u, 52u, 64u, 80u, 96u, 128u, 160u, 208u, 256u, 320u, 416u, 512u, 640u, 832u, 1024u, 1280u, PG_MAX})
+        if (pages <= double(c)) return c;
+    return PG_MAX + 1;
+}
+
+struct PageShape {
+    uint32_t cap, buckets, queue, words, warps, blocks, groups;  // blocks, groups: per SM
+    size_t smem;
+};
+
+// The map of a group and the warps that share it: one while the maps leave an SM sixteen
+// warps, since warps that share a ball wait for each other at every round, else the fewest
+// that give it 24, and never more than a round of the ball has items for.  Measured with
+// 1 / 2 / 4 / 8 / 16 warps, ms a call: 1.07M-node join (balls of up to 50 pages) 1.45 / 1.87 /
+// 2.35 / 3.57 / 6.6; 264k-node join (80 pages) 0.95 / 0.93 / 0.95 / 1.26 / 2.0; balls of up to
+// 190 pages 3.5 / 2.2 / 1.7 / 1.8 / 2.5, and 1.6 with eight where four warps make 16 of an SM.
+static PageShape page_shape(uint32_t cap, uint32_t items, int sms, bool hier) {
+    PageShape p{};
+    p.cap = cap;
+    p.buckets = 32;
+    while (p.buckets < cap) p.buckets *= 2;
+    p.queue = std::min<uint32_t>(std::max<uint32_t>(4 * cap, 64), 2048);
+    p.words = (32 * cap + 2 * p.buckets + cap + p.queue + PC_WORDS + 3) / 4 * 4;
+    const uint32_t want = std::max<uint32_t>(1, (items + sms - 1) / sms);  // sources per SM
+    const uint32_t most = cap <= 32 ? 2 : cap <= 100 ? 4 : cap <= 300 ? 8 : cap <= 700 ? 16 : 32;
+    for (uint32_t W = 1;; W *= 2) {
+        const uint32_t G = pg_groups(int(W));
+        p.warps = W;
+        p.smem = size_t(p.words) * 4 * G;
+        p.blocks = std::min<uint32_t>(uint32_t(233472 / (p.smem + 1024 + 640)), W == 1 ? 8 : 32 / W);
+        p.groups = p.blocks * G;
+        if (hier ? (W == 4 || (W == 1 && cap <= 96)) : p.blocks && (W >= most || W * std::min(p.groups, want) >= (W == 1 ? 16u : 24u))) break;
+    }
+    if (!p.blocks) fail(RN_EINTERNAL, "a group's pages do not fit an SM");
+    return p;
+}
+
+template <int W, bool HIER>
+static void launch_pages(const SearchArgs &a, const PageShape &p, uint32_t grid, cudaStream_t st) {
+    static std::once_flag once[MAX_DEVICES];
+    std::call_once(once[attr_device()], [&] {
+        RN_CUDA(cudaFuncSetAttribute(k_source_search<W, HIER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 231424));
+        RN_CUDA(cudaFuncSetAttribute(k_source_search<W, HIER>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    });
+    k_source_search<W, HIER><<<grid, 32 * W * pg_groups(W), p.smem, st>>>(a);
+    RN_CUDA(cudaGetLastError());
+}
+
+// One launch of the search by pages over `items` sources.
+static void page_launch(const DeviceGraph &g, uint32_t cap, SearchArgs a, uint32_t items, Workspace *ws, cudaStream_t st,
+                        bool hier) {
+    const PageShape p = page_shape(cap, items, ws->num_sms, hier);
+    if (!g.ell) fail(RN_EINTERNAL, "search by pages without rows");
+    a.ell = g.ell;
+    a.n_rows = uint32_t(g.n + g.nvirt);
+    a.pg_cap = p.cap;
+    a.pg_buckets = p.buckets;
+    a.pg_queue = p.queue;
+    a.pg_words = p.words;
+    a.pg_resident = std::max<uint32_t>(p.groups, 1);
+    const uint32_t G = pg_groups(int(p.warps));
+    const uint32_t grid = std::max<uint32_t>(1, std::min<uint32_t>((items + G - 1) / G, uint32_t(ws->num_sms) * p.blocks));
+    if (hier) {
+        if (p.warps == 1) launch_pages<1, true>(a, p, grid, st);
+        else launch_pages<4, true>(a, p, grid, st);
+    } else {
+        switch (p.warps) {
+            case 1: launch_pages<1, false>(a, p, grid, st); break;
+            case 2: launch_pages<2, false>(a, p, grid, st); break;
+            case 4: launch_pages<4, false>(a, p, grid, st); break;
+            case 8: launch_pages<8, false>(a, p, grid, st); break;
+            case 16: launch_pages<16, false>(a, p, grid, st); break;
+            default: launch_pages<32, false>(a, p, grid, st); break;
+        }
+    }
+    ws->launches++;
+}
+
 // One warp-search launch over `items` sources with maps of ms slots: a block per
 // src_warps sources up to three blocks per SM of the device.  The warp search uses no slab,
 // so a server's request is not held to the slab regions it was given (those serve its
 // tile fallback): its blocks share the SMs with the other requests' as they free up.
-static void source_launch(uint32_t ms, SearchArgs a, uint32_t items, Workspace *ws, cudaStream_t st,
-                          bool hier = false) {
+static void hash_launch(uint32_t ms, SearchArgs a, uint32_t items, Workspace *ws, cudaStream_t st,
+                        bool hier = false) {
     a.H = ms;
     a.hshift = 32 - log2u(ms);
     a.max_fill = ms * 7 / 8;
@@ -3029,6 +3838,14 @@ static double predicted_ball(const Workspace *ws, uint32_t theta) {
     return double(ws->ball_max) * r * r;
 }
 
+// One source-search launch over `items` sources: by pages (size: pages of a group's map) or
+// by hashed nodes (size: slots of a warp's map).
+static void source_launch(const DeviceGraph &g, bool paged, uint32_t size, const SearchArgs &a, uint32_t items,
+                          Workspace *ws, cudaStream_t st, bool hier = false) {
+    if (paged) page_launch(g, size, a, items, ws, st, hier);
+    else hash_launch(size, a, items, ws, st, hier);
+}
+
 // The ball of a source at bound theta on a graph with no search behind it yet: on a
 // planar road network the nodes within theta are about those within theta / w_med hops,
 // and a lattice holds 2 r^2 nodes within r hops; never more than the graph.
@@ -3047,7 +3864,7 @@ static bool use_source_search(const DeviceGraph &g, const Workspace *ws, const E
     if (cfg.tile_width == 1) return true;
     if (cfg.tile_width || cfg.map_slots) return false;
     const double ball = ws->ball_theta ? predicted_ball(ws, theta) : first_ball_estimate(g, theta, median_w);
-    return ball <= src_fit(SRC_MS_MAX);
+    return ball <= (by_pages(g, theta) ? PG_BALL_MAX : src_fit(SRC_MS_MAX));
 }
 
 // First warp map: the smallest whose 7/8 holds 1.3 times the predicted mean ball and
@@ -3056,8 +3873,20 @@ static bool use_source_search(const DeviceGraph &g, const Workspace *ws, const E
 // no history: the smallest map that fits the ball estimated from the bound (`first`, the
 // largest ball a lattice would give: k closest pairs, whose searches teach the workspace
 // nothing), else 2048 slots (a join's first search, which its measured balls then size).
-static uint32_t source_first_map(const Workspace *ws, uint32_t theta, double first = 0) {
+static uint32_t source_first_map(const DeviceGraph &g, const Workspace *ws, uint32_t theta, double first = 0) {
     const double b = predicted_ball(ws, theta);
+    if (by_pages(g, theta)) {
+        // the most pages the last search met (they grow a little slower than the ball: up
+        // with the squared radius, down with its 1.5th power) and a little room, since other
+        // sources reach a few more; with no history, the estimated ball at half-full pages,
+        // else 96 pages (a join's first search, which its measured balls then size)
+        double p = first > 0 ? first / 16 + 16 : 96;
+        if (b > 0 && ws->page_max > 0) {
+            const double r = double(theta) / double(ws->ball_theta);
+            p = ws->page_max * (r > 1 ? r * r : std::pow(r, 1.5)) * 1.06 + 2;
+        }
+        return page_cap(g, p);
+    }
     if (b <= 0) {
         if (first <= 0) return 2048;
         for (uint32_t ms = SRC_MS_MIN; ms <= SRC_MS_MAX; ms *= 2)
@@ -3092,13 +3921,14 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
     ensure_ranges(&ws->failed2, &ws->failed2_cap, std::max<uint32_t>(nsrc, 1));
     a.failed = ws->failed;
     RN_CUDA(cudaEventRecord(ws->evs0, st));
-    if (nsrc) source_launch(ms0, a, nsrc, ws, st);
+    const bool paged = by_pages(g, theta);
+    if (nsrc) source_launch(g, paged, ms0, a, nsrc, ws, st);
     RN_CUDA(cudaEventRecord(ws->evs1, st));
     Control c = read_control(ws, st);
     ws->retry_ms = 0;
     ws->src_tiles = false;
-    ws->blocks_per_sm = nsrc ? source_blocks_per_sm(ms0) : 0;
-    double ball = c.src_max_ball;
+    ws->blocks_per_sm = !nsrc ? 0 : paged ? int(page_shape(ms0, nsrc, ws->num_sms, false).blocks) : source_blocks_per_sm(ms0);
+    double ball = c.src_max_ball, pages = c.src_max_pages;
     // mean ball of the sources the first pass completed (0 when none did)
     const double mean = nsrc > c.n_failed ? double(c.slots) / double(nsrc - c.n_failed) : 0.0;
     auto learn = [&] {
@@ -3107,6 +3937,7 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
             ws->ball_theta = std::max<uint32_t>(theta, 1);
             ws->ball_max = ball;
             ws->ball_mean = mean;
+            ws->page_max = pages;
         }
     };
     if (!c.n_failed || c.err || c.check[0]) {
@@ -3124,6 +3955,19 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
     auto route = [&](const uint4 &f, uint32_t failed_at) {
         const double e = estimate(f);
         ball = std::max(ball, e);
+        if (paged) {
+            // its pages, in proportion to the nodes met when they were used up
+            const double need = double(failed_at) * std::max(1.3, 1.15 * e / double(std::max<uint32_t>(f.w, 1)));
+            const uint32_t size = page_cap(g, page_class(need));
+            if (size > failed_at && need <= 1.3 * PG_MAX) {
+                pages = std::max<double>(pages, std::min(need, double(PG_MAX)));
+                grow[size].push_back(make_uint4(f.x, 0, 0, 0));
+            } else {
+                to_tiles.push_back(f);
+                tile_est = std::max(tile_est, e);
+            }
+            return;
+        }
         uint32_t ms = failed_at * 2;
         while (ms <= SRC_MS_MAX && e > src_fit(ms)) ms *= 2;
         if (ms <= SRC_MS_MAX) {
@@ -3145,11 +3989,12 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
         SearchArgs r = a;
         r.range_list = ws->failed2;
         r.ntiles = n;
-        source_launch(ms, r, n, ws, st);
+        source_launch(g, paged, ms, r, n, ws, st);
         *retried += n;
         c = read_control(ws, st);
         if (c.err || c.check[0]) return c;
         ball = std::max<double>(ball, c.src_max_ball);
+        pages = std::max<double>(pages, c.src_max_pages);
         for (const uint4 &f : read_ranges(ws->failed, c.n_failed, st)) route(f, ms);
     }
     ws->src_tiles = !to_tiles.empty();
@@ -3397,7 +4242,7 @@ void run_join(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint
     ensure_ranges(&ws->failed, &ws->failed_cap, std::max<uint32_t>(ntiles, 1));
     ensure_ranges(&ws->failed2, &ws->failed2_cap, std::max<uint32_t>(ntiles, 1));
     ensure_pairs(ws, std::max<uint64_t>(ws->pair_cap, uint64_t(nR) * 64));
-    const uint32_t ms0 = by_source ? source_first_map(ws, theta) : 0;
+    const uint32_t ms0 = by_source ? source_first_map(g, ws, theta) : 0;
 
     const uint32_t vbits = bits_for(g.n);
     SearchArgs a{};
@@ -3575,7 +4420,7 @@ void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg
         if (cfg.tile_src) tile_src = std::min(cfg.tile_src, T);
     }
     if (by_source) tile_src = 1;
-    const uint32_t ms0 = by_source ? source_first_map(ws, max_bound) : 0;
+    const uint32_t ms0 = by_source ? source_first_map(g, ws, max_bound) : 0;
     std::vector<uint4> ranges;
     for (uint32_t i = 0; i < nq; i++)
         for (uint32_t j = 0; j < nsrc[i]; j += tile_src)
@@ -4075,7 +4920,7 @@ void run_kcp(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint3
         if (by_source) {
             a.tile_src = 1;
             c = source_search_all(g, ws, a, nR,
-                                  source_first_map(ws, uint32_t(tau), first_ball_estimate(g, uint32_t(tau), median_w)), T,
+                                  source_first_map(g, ws, uint32_t(tau), first_ball_estimate(g, uint32_t(tau), median_w)), T,
                                   uint32_t(tau), {}, st,
                                   &retried, false);
         } else {
@@ -4235,10 +5080,36 @@ struct PointsState {
 void points_destroy(PointsState *ps) {
     if (!ps) return;
     for (void *p : {(void *)ps->aug.row_ptr, (void *)ps->aug.adj, (void *)ps->aug.perm, (void *)ps->aug.iperm,
-                    (void *)ps->ids, (void *)ps->keys, (void *)ps->found, (void *)ps->patches})
+                    (void *)ps->aug.ell, (void *)ps->ids, (void *)ps->keys, (void *)ps->found, (void *)ps->patches})
         device_free(p);
     workspace_destroy(ps->ws);
     delete ps;
+}
+
+// The arcs that lead to an edge's first and last point, in the search's rows (a node's arc
+// j sits in its row, or behind the row's last slot in its overflow rows).
+__global__ void k_rows_patch(const uint32_t *__restrict__ row_ptr, uint32_t n, const uint4 *__restrict__ patches,
+                             uint32_t count, uint2 *rows) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+        const uint4 p = patches[i];  // arc position, new column, new weight, the arc's node
+        if (p.w >= n) continue;
+        uint32_t j = p.x - row_ptr[p.w], left = row_ptr[p.w + 1] - row_ptr[p.w], row = p.w;
+        if (j >= left) continue;
+        while (left > PG_ROW && j >= PG_ROW - 1) {  // on in the node's overflow row
+            row = rows[size_t(row) * PG_ROW + PG_ROW - 1].x;
+            j -= PG_ROW - 1;
+            left -= PG_ROW - 1;
+        }
+        rows[size_t(row) * PG_ROW + j] = make_uint2(p.y, p.z);
+    }
+}
+
+// The point nodes' rows: two links each (adjacency entries 2 i and 2 i + 1).
+__global__ void k_rows_points(const uint2 *__restrict__ links, uint32_t count, uint32_t n, uint2 *rows) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count * PG_ROW; i += gridDim.x * blockDim.x) {
+        const uint32_t k = i % PG_ROW;
+        rows[size_t(n) * PG_ROW + i] = k < 2 ? links[2 * (i / PG_ROW) + k] : make_uint2(n + i / PG_ROW, PG_PAD);
+    }
 }
 
 // Build the subdivided graph for the points in ps->aug (grow-only buffers).
@@ -4334,13 +5205,14 @@ static void points_graph(const DeviceGraph &g, const std::vector<uint32_t> &perm
             tail[4 * size_t(me) + 2] = next;
             tail[4 * size_t(me) + 3] = next_pos - pos[i];
         }
-        patches.push_back(make_uint4(f.x, node[order[j]], pos[order[j]], 0));            // p -> o_1
-        patches.push_back(make_uint4(f.y, node[order[e - 1]], w - pos[order[e - 1]], 0));  // q -> o_k
+        patches.push_back(make_uint4(f.x, node[order[j]], pos[order[j]], p));            // p -> o_1
+        patches.push_back(make_uint4(f.y, node[order[e - 1]], w - pos[order[e - 1]], q));  // q -> o_k
         j = e;
     }
     // the subdivided graph's arrays
     if (ps->cap_nodes < n_aug || ps->cap_arcs < arcs_aug) {
-        for (void **q : {(void **)&ps->aug.row_ptr, (void **)&ps->aug.adj, (void **)&ps->aug.perm, (void **)&ps->aug.iperm}) {
+        for (void **q : {(void **)&ps->aug.row_ptr, (void **)&ps->aug.adj, (void **)&ps->aug.perm, (void **)&ps->aug.iperm,
+                         (void **)&ps->aug.ell}) {
             device_free(*q);
             *q = nullptr;
         }
@@ -4350,6 +5222,7 @@ static void points_graph(const DeviceGraph &g, const std::vector<uint32_t> &perm
         ps->aug.adj = (uint32_t *)device_alloc(ps->cap_arcs * 8);
         ps->aug.perm = (uint32_t *)device_alloc(ps->cap_nodes * 4);
         ps->aug.iperm = (uint32_t *)device_alloc(ps->cap_nodes * 4);
+        if (g.paged) ps->aug.ell = (uint4 *)device_alloc((ps->cap_nodes + g.nvirt) * PG_ROW * 8);
         workspace_destroy(ps->ws);
         ps->ws = nullptr;
         DeviceGraph capg{};
@@ -4358,6 +5231,9 @@ static void points_graph(const DeviceGraph &g, const std::vector<uint32_t> &perm
     }
     ps->aug.n = uint32_t(n_aug);
     ps->aug.arcs = arcs_aug;
+    ps->aug.nvirt = g.nvirt;
+    ps->aug.paged = g.paged && n_aug + g.nvirt <= PG_ROWS_MAX;
+    ps->aug.far = g.far;  // (a path crosses an edge's links at most once: no longer than over whole edges)
     std::vector<uint32_t> rp_tail(np), perm_tail(np);
     for (uint32_t i = 0; i < np; i++) {
         rp_tail[i] = uint32_t(g.arcs + 2ull * (i + 1));  // row_ptr[n + 1 + i]
@@ -4376,6 +5252,17 @@ static void points_graph(const DeviceGraph &g, const std::vector<uint32_t> &perm
         RN_CUDA(cudaMemcpyAsync(ps->patches, patches.data(), patches.size() * 16, cudaMemcpyHostToDevice, st));
         k_patch_arcs<<<std::min<uint32_t>((uint32_t(patches.size()) + 255) / 256, 1024), 256, 0, st>>>(
             reinterpret_cast<uint2 *>(ps->aug.adj), ps->patches, uint32_t(patches.size()), g.arcs);
+        RN_CUDA(cudaGetLastError());
+    }
+    if (ps->aug.paged) {
+        // the search's rows: the graph's, the patched arcs, the point nodes' two links
+        rows_copy(g, 0, uint32_t(n_aug), ps->aug.ell, st);
+        if (np) {
+            k_rows_patch<<<std::min<uint32_t>((uint32_t(patches.size()) + 255) / 256, 1024), 256, 0, st>>>(
+                g.row_ptr, g.n, ps->patches, uint32_t(patches.size()), reinterpret_cast<uint2 *>(ps->aug.ell));
+            k_rows_points<<<std::min<uint32_t>((np * PG_ROW + 255) / 256, 4096), 256, 0, st>>>(
+                reinterpret_cast<const uint2 *>(ps->aug.adj) + g.arcs, np, g.n, reinterpret_cast<uint2 *>(ps->aug.ell));
+        }
         RN_CUDA(cudaGetLastError());
     }
     // the query's sets: the point nodes
@@ -4817,6 +5704,9 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
     for (uint32_t m = SRC_MS_MIN; m <= SRC_MS_MAX && !map_slots; m *= 2)
         if (double(max_part) <= src_fit(m)) map_slots = m;
     if (!map_slots) fail(RN_EINVAL, "the hierarchical variant takes parts of at most 6516 nodes");
+    // by pages: the part's consecutive ids, and its overflow rows' (consecutive too)
+    const uint32_t part_virt = uint32_t(std::min<uint64_t>(g.nvirt, uint64_t(max_part) * g.row_chain));
+    const uint32_t part_pages = std::max<uint32_t>(8, (max_part + 31) / 32 + (part_virt + 31) / 32 + 2);
     std::lock_guard<std::mutex> device_lock(ws->sh->mu);
     Range range("rn.hier");
     *stats = rn_query_stats{};
@@ -4936,7 +5826,7 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
             a.brd_d = brd_d;
             a.brd_cap = brd_cap;
             a.brd_count = h->count;
-            if (nR) source_launch(map_slots, a, nR, ws, st, true);
+            if (nR) source_launch(g, by_pages(g, bnd), by_pages(g, bnd) ? part_pages : map_slots, a, nR, ws, st, true);
             c = read_control(ws, st);
             counts();
             check_control(c);
@@ -5043,7 +5933,7 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
             a.tile_inst = ti;
             a.slab = ws->sh->slab;
             const Control cc =
-                source_search_all(g, ws, a, nf, source_first_map(ws, bnd), 32, bnd, {}, st, &retried, false);
+                source_search_all(g, ws, a, nf, source_first_map(g, ws, bnd), 32, bnd, {}, st, &retried, false);
             check_control(cc);
             if (cc.pairs > hit_cap) {
                 hit_cap = cc.pairs + cc.pairs / 4;
@@ -5253,7 +6143,8 @@ uint32_t plan_tile_src(const BatchPlan &p) { return std::max<uint32_t>(1, p.T / 
 
 // The smallest warp map whose 7/8 holds a ball of `ball` nodes with room to spare, or 0
 // when even the largest does not.
-uint32_t warp_map_for_ball(double ball) {
+uint32_t warp_map_for_ball(double ball, bool paged) {
+    if (paged) return page_class(ball) <= PG_MAX ? page_class(ball) : 0;  // (the ball's pages)
     for (uint32_t ms = SRC_MS_MIN; ms <= SRC_MS_MAX; ms *= 2)
         if (ball <= src_fit(ms)) return ms;
     return 0;
@@ -5346,7 +6237,9 @@ struct Batch {
     std::vector<double> tile_cost;   // per instance: SM cycles of one of its tiles, last run
     bool costs_known = false;        // tile_cost holds measurements (else a size proxy)
     bool laid_out_by_cost = false;   // the layout used measured costs
-    DeviceGraph ug;  // the union graph (row_ptr, adj, iperm)
+    DeviceGraph ug;  // the union graph (row_ptr, adj, iperm, rows)
+    bool paged = false;        // its sources are searched by pages
+    uint32_t theta_max = 0;    // the largest bound of an instance
     uint32_t *sbits = nullptr, *node_off_d = nullptr, *inst_ball = nullptr;
     uint8_t *inst_swap = nullptr;  // per instance: searched from S (null when none is)
     Workspace *ws = nullptr;  // control block, retry lists, global maps, events of the batch
@@ -5392,7 +6285,7 @@ void batch_destroy(Batch *b) {
     for (void *p : {(void *)b->sbits, (void *)b->inst_swap, (void *)b->node_off_d, (void *)b->inst_ball, (void *)b->inst_pairs,
                     (void *)b->inst_cycles, (void *)b->pair_off_d, (void *)b->keyA, (void *)b->keyB,
                     (void *)b->valA, (void *)b->valB, (void *)b->hist, (void *)b->out_u, (void *)b->out_v,
-                    (void *)b->out_d, (void *)b->ug.row_ptr, (void *)b->ug.adj, (void *)b->ug.iperm})
+                    (void *)b->out_d, (void *)b->ug.row_ptr, (void *)b->ug.adj, (void *)b->ug.iperm, (void *)b->ug.ell})
         device_free(p);
     if (b->stream) cudaStreamDestroy(b->stream);
     workspace_destroy(b->ws);
@@ -5414,12 +6307,12 @@ static bool batch_adapt_maps(Batch *b) {
     bool changed = false;
     for (uint32_t i = 0; i < b->nq; i++) {
         const bool measured = b->ball_T[i] == b->plan[i].T;
-        if (b->plan[i].T == 1 && measured && !warp_map_for_ball(b->ball[i])) {
+        if (b->plan[i].T == 1 && measured && !warp_map_for_ball(b->ball[i], b->paged)) {
             b->plan[i] = BIG_PLAN;
             changed = true;
         }
         uint32_t m;
-        if (b->plan[i].T == 1) m = measured ? warp_map_for_ball(b->ball[i]) : 2048;
+        if (b->plan[i].T == 1) m = measured ? warp_map_for_ball(b->ball[i], b->paged) : b->paged ? 96 : 2048;
         else m = b->ball_T[i] == b->plan[i].T ? map_for_ball(b->ball[i]) : SMEM_H;
         if (m != b->map[i]) changed = true;
         b->map[i] = m;
@@ -5593,7 +6486,7 @@ static void batch_launch_group(Batch *b, const Batch::Group &g, cudaStream_t st)
     a.n_nodes = b->ug.n;
     a.n_arcs = b->ug.arcs;
     if (g.T == 1) {  // the warp search: one source per tile, a warp map of g.map slots
-        source_launch(g.map, a, g.nsrc, b->ws, st);
+        source_launch(b->ug, b->paged, g.map, a, g.nsrc, b->ws, st);
         return;
     }
     if (g.map > SMEM_HW) {
@@ -5619,7 +6512,7 @@ static uint64_t batch_run_eager(Batch *b, cudaStream_t st) {
         for (const auto &g : b->groups) {
             RN_CUDA(cudaMemsetAsync(&b->ws->ctl->tile_next, 0, 8, st));  // tile_next, n_failed
             if (g.T == 1)
-                c = source_search_all(b->ug, b->ws, batch_args(b, g), g.nsrc, g.map, TILE_PLAN.T, RN_THETA_MAX, {},
+                c = source_search_all(b->ug, b->ws, batch_args(b, g), g.nsrc, g.map, TILE_PLAN.T, b->theta_max, {},
                                       st, &retried, false);
             else
                 c = search_all(b->ug, b->ws, g.T, batch_args(b, g), g.tiles, st, &retried, g.map, false);
@@ -5845,7 +6738,18 @@ Batch *batch_create(const std::vector<const DeviceGraph *> &graphs, const std::v
         b->ball_T.assign(b->nq, 0);
         b->tile_cost.resize(b->nq);
         for (uint32_t i = 0; i < b->nq; i++) b->tile_cost[i] = double(graphs[i]->n);  // until measured
-        uint64_t nsum = 0, asum = 0;
+        uint64_t nsum = 0, asum = 0, vsum = 0;
+        b->paged = b->nq > 0;
+        for (uint32_t i = 0; i < b->nq; i++) {
+            const uint32_t th = theta[i] == RN_INF ? RN_THETA_MAX : theta[i];
+            b->paged = b->paged && by_pages(*graphs[i], th);
+            b->theta_max = std::max(b->theta_max, std::min(th, RN_THETA_MAX));
+            b->ug.far = std::max(b->ug.far, graphs[i]->far);
+            nsum += graphs[i]->n;
+            vsum += graphs[i]->nvirt;
+        }
+        b->paged = b->paged && nsum + 1 + vsum <= PG_ROWS_MAX && (b->theta_max <= PG_BOUND_MAX || b->ug.far <= PG_BOUND_MAX);
+        nsum = 0;
         for (uint32_t i = 0; i < b->nq; i++) {
             b->n[i] = graphs[i]->n;
             b->theta[i] = theta[i] == RN_INF ? RN_THETA_MAX : theta[i];
@@ -5854,7 +6758,8 @@ Batch *batch_create(const std::vector<const DeviceGraph *> &graphs, const std::v
             // the default plan: the warp search while the ball estimated from the bound
             // fits a 2048-slot warp map (a dozen warps per SM or more), else tiles, whose
             // sources share their searches' passes
-            if (graphs[i]->n < SK_NODE && first_ball_estimate(*graphs[i], b->theta[i], median_w[i]) <= src_fit(2048))
+            if (graphs[i]->n < SK_NODE &&
+                first_ball_estimate(*graphs[i], b->theta[i], median_w[i]) <= (b->paged ? PG_BALL_MAX : src_fit(2048)))
                 b->plan[i] = WARP_PLAN;
             b->node_off[i] = uint32_t(nsum);
             nsum += graphs[i]->n;
@@ -5885,6 +6790,22 @@ Batch *batch_create(const std::vector<const DeviceGraph *> &graphs, const std::v
         b->ug.row_ptr = (uint32_t *)device_alloc((size_t(b->n_u) + 1) * 4);
         b->ug.adj = (uint32_t *)device_alloc(std::max<uint64_t>(asum, 1) * 8);
         b->ug.iperm = (uint32_t *)device_alloc(size_t(b->n_u) * 4);
+        if (b->paged) {
+            b->ug.paged = true;
+            b->ug.nvirt = uint32_t(vsum);
+            b->ug.ell = (uint4 *)device_alloc((size_t(b->n_u) + vsum) * PG_ROW * 8);
+            uint64_t voff = b->n_u;
+            for (uint32_t i = 0; i < b->nq; i++) {
+                const DeviceGraph &g = *graphs[i];
+                rows_copy(g, b->node_off[i], uint32_t(voff), b->ug.ell, b->stream);
+                voff += g.nvirt;
+            }
+            const uint2 none = make_uint2(b->pad, PG_PAD);  // the pad node: no arcs
+            const std::vector<uint2> pad_row(PG_ROW, none);
+            RN_CUDA(cudaMemcpyAsync(b->ug.ell + size_t(b->pad) * (PG_ROW / 2), pad_row.data(), PG_ROW * 8,
+                                    cudaMemcpyHostToDevice, b->stream));
+            RN_CUDA(cudaStreamSynchronize(b->stream));
+        }
         uint64_t aoff = 0;
         for (uint32_t i = 0; i < b->nq; i++) {
             const DeviceGraph &g = *graphs[i];

@@ -68,6 +68,13 @@ struct DeviceGraph {
     uint32_t *iperm = nullptr;    // internal id -> original id
     bool iperm_inverts_perm = true;  // false when output ids are not the input ids (points)
     bool symmetric = false;          // every arc has its reverse with the same weight (undirected)
+    // the source search's rows: eight arc slots (col, w) per node, a node with more arcs
+    // going on in overflow rows n, n + 1, ... (nvirt of them; at most row_chain per node);
+    // paged: the ids have the locality the search by pages wants; far: no distance is longer
+    uint4 *ell = nullptr;
+    uint32_t nvirt = 0, row_chain = 0;
+    bool paged = false;
+    uint64_t far = 0;
     // node coordinates (rn_graph_load's xy), or none: per node (x, y) by internal id, and
     // the leaves of the partition -- leaf i holds internal ids [leaf_start[i],
     // leaf_start[i + 1]) -- with their bounding rectangles (xmin, ymin, xmax, ymax)

@@ -3716,7 +3716,11 @@ struct PageShape {
     size_t smem;
 };
 
-// The map of a group and the warps that share it: one while the maps leave an SM sixteen
+// The map of a group and the warps that share it.  Two buckets of two entries a page: a page
+// displaced from its home bucket stops a step's 128 arc slots for a probe, and at one bucket a
+// page (1% of the pages displaced) that cost 2.06 ms against 1.70 with balls of 190 pages, 0.94
+// against 0.90 on the 264k-node join; four buckets a page cost an SM more groups than they
+// save.  The warps: one while the maps leave an SM sixteen
 // warps, since warps that share a ball wait for each other at every round, else the fewest
 // that give it 24, and never more than a round of the ball has items for.  Measured with
 // 1 / 2 / 4 / 8 / 16 warps, ms a call: 1.07M-node join (balls of up to 50 pages) 1.45 / 1.87 /
@@ -3726,7 +3730,7 @@ static PageShape page_shape(uint32_t cap, uint32_t items, int sms, bool hier) {
     PageShape p{};
     p.cap = cap;
     p.buckets = 32;
-    while (p.buckets < cap) p.buckets *= 2;
+    while (p.buckets < 2 * cap && p.buckets < 2048) p.buckets *= 2;
     p.queue = std::min<uint32_t>(std::max<uint32_t>(4 * cap, 64), 2048);
     p.words = (32 * cap + 2 * p.buckets + cap + p.queue + PC_WORDS + 3) / 4 * 4;
     const uint32_t want = std::max<uint32_t>(1, (items + sms - 1) / sms);  // sources per SM
@@ -3846,6 +3850,15 @@ static void source_launch(const DeviceGraph &g, bool paged, uint32_t size, const
     else hash_launch(size, a, items, ws, st, hier);
 }
 
+// The most pages of a ball at bound theta, from the last searches by pages on this workspace
+// (pages grow a little slower than balls: up with the squared radius, down with its 1.5th
+// power), 0 when there was none.
+static double pages_at(const Workspace *ws, uint32_t theta) {
+    if (!ws->ball_theta || ws->page_max <= 0) return 0;
+    const double r = double(theta) / double(ws->ball_theta);
+    return ws->page_max * (r > 1 ? r * r : std::pow(r, 1.5));
+}
+
 // The ball of a source at bound theta on a graph with no search behind it yet: on a
 // planar road network the nodes within theta are about those within theta / w_med hops,
 // and a lattice holds 2 r^2 nodes within r hops; never more than the graph.
@@ -3876,16 +3889,11 @@ static bool use_source_search(const DeviceGraph &g, const Workspace *ws, const E
 static uint32_t source_first_map(const DeviceGraph &g, const Workspace *ws, uint32_t theta, double first = 0) {
     const double b = predicted_ball(ws, theta);
     if (by_pages(g, theta)) {
-        // the most pages the last search met (they grow a little slower than the ball: up
-        // with the squared radius, down with its 1.5th power) and a little room, since other
-        // sources reach a few more; with no history, the estimated ball at half-full pages,
-        // else 96 pages (a join's first search, which its measured balls then size)
-        double p = first > 0 ? first / 16 + 16 : 96;
-        if (b > 0 && ws->page_max > 0) {
-            const double r = double(theta) / double(ws->ball_theta);
-            p = ws->page_max * (r > 1 ? r * r : std::pow(r, 1.5)) * 1.06 + 2;
-        }
-        return page_cap(g, p);
+        // the most pages the last searches met and a little room, since other sources reach a
+        // few more; with no history, the estimated ball at half-full pages, else 96 pages (a
+        // join's first search, which its measured balls then size)
+        const double seen = pages_at(ws, theta);
+        return page_cap(g, seen > 0 ? seen * 1.06 + 2 : first > 0 ? first / 16 + 16 : 96);
     }
     if (b <= 0) {
         if (first <= 0) return 2048;
@@ -3934,10 +3942,13 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
     auto learn = [&] {
         // (k closest pairs lowers its bound as it goes: its balls say nothing of theta)
         if (learn_balls && nsrc && ball >= 64) {  // a handful of nodes says little about the growth
+            // (the most pages of the last searches, scaled to this bound: other sets' largest
+            // balls differ by some percent, and a map too small costs a second launch)
+            const double was = pages_at(ws, theta);
             ws->ball_theta = std::max<uint32_t>(theta, 1);
             ws->ball_max = ball;
             ws->ball_mean = mean;
-            ws->page_max = pages;
+            ws->page_max = std::max(pages, 0.97 * was);
         }
     };
     if (!c.n_failed || c.err || c.check[0]) {

@@ -29,6 +29,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <string>
@@ -228,6 +229,7 @@ void upload_geometry(const float *xy, const std::vector<uint32_t> &order, const 
 struct Control {
     uint32_t err;          // 1: id >= n, 2: repeated id or R/S overlap
     uint32_t r_count;      // R nodes after validation
+    uint32_t place_next;   // blocks of the placement started
     uint32_t tile_next;    // work-queue head of the persistent search
     uint32_t n_failed;     // tiles whose slab overflowed
     unsigned long long pairs;
@@ -246,7 +248,10 @@ struct Control {
     uint32_t src_max_ball;          // largest ball of a source the warp search completed
     uint32_t max_seg;               // most pairs one source emitted in the warp search
     uint32_t src_max_pages;         // most pages of a ball the source search completed
-    unsigned long long pages;       // sum over those balls of their pages
+    // the source search's counters: every block adds its sums to one of the copies (all
+    // blocks end at about the same time, and a counter's one address takes one addition
+    // after another); read_control adds them up into the fields above
+    unsigned long long tel[16][16];
 };
 
 // Record the first failed device-side check (the access it guarded is skipped).
@@ -301,7 +306,9 @@ struct Workspace {
     uint32_t rsorted_cap = 0;
     uint4 *failed = nullptr, *failed2 = nullptr;  // source ranges whose map overflowed, to search again
     uint32_t failed_cap = 0, failed2_cap = 0;
-    Control *ctl = nullptr;
+    Control *ctl = nullptr;      // then, in the same allocation, the three bitmaps
+    size_t clear_bytes = 0;
+    uint32_t *ctl_words(size_t at) const { return reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(ctl) + at); }
     Control *ctl_host = nullptr;  // pinned
     struct DeviceShared *sh = nullptr;  // the device's slab, shared by every graph on it
     uint32_t *kcp = nullptr;     // k closest pairs: histogram, live threshold, select state
@@ -335,6 +342,10 @@ struct Workspace {
     // handed sources to the tile search (their pairs are then not in segments)
     uint2 *seg = nullptr;
     uint32_t seg_cap = 0;
+    bool src_clean = false;  // its first launch completed every source
+    // the placement's look-back words (epoch, kind, count), one per block
+    unsigned long long *place_state = nullptr;
+    uint32_t place_cap = 0, place_epoch = 0;
     uint32_t *slist = nullptr;  // the warp search's per-warp lists of S nodes (SRC_LIST_WORDS)
     bool src_tiles = false;
     uint32_t launches = 0;  // kernels launched by the current query
@@ -357,11 +368,14 @@ Workspace *workspace_create(const DeviceGraph &g) {
         ws->sh = &g_shared[dev];
         ws->n = g.n;
         ws->nwords = (g.n + 31) / 32;
-        ws_alloc(ws, (void **)&ws->used_bits, size_t(ws->nwords) * 4);
-        ws_alloc(ws, (void **)&ws->rbits, size_t(ws->nwords) * 4);
-        ws_alloc(ws, (void **)&ws->sbits, size_t(ws->nwords) * 4);
+        // the control block and the bitmaps in one piece: one clear per query
+        const size_t head = (sizeof(Control) + 255) / 256 * 256, bits = (size_t(ws->nwords) * 4 + 255) / 256 * 256;
+        ws->clear_bytes = head + 3 * bits;
+        ws_alloc(ws, (void **)&ws->ctl, ws->clear_bytes);
+        ws->used_bits = ws->ctl_words(head);
+        ws->rbits = ws->ctl_words(head + bits);
+        ws->sbits = ws->ctl_words(head + 2 * bits);
         ws_alloc(ws, (void **)&ws->block_sums, (ws->nwords / 1024 + 2) * 4);
-        ws_alloc(ws, (void **)&ws->ctl, sizeof(Control));
         RN_CUDA(cudaMallocHost(&ws->ctl_host, sizeof(Control)));
         RN_CUDA(cudaEventCreate(&ws->ev0));
         RN_CUDA(cudaEventCreate(&ws->ev1));
@@ -377,9 +391,6 @@ Workspace *workspace_create(const DeviceGraph &g) {
 
 void workspace_destroy(Workspace *ws) {
     if (!ws) return;
-    device_free(ws->used_bits);
-    device_free(ws->rbits);
-    device_free(ws->sbits);
     device_free(ws->block_sums);
     device_free(ws->rsorted);
     device_free(ws->failed);
@@ -402,6 +413,7 @@ void workspace_destroy(Workspace *ws) {
         device_free(p);
     device_free(ws->own_gmap);
     device_free(ws->seg);
+    device_free(ws->place_state);
     device_free(ws->slist);
     if (ws->own_sh) {
         device_free(ws->own_sh->gretry);
@@ -444,27 +456,26 @@ static void grow(Workspace *ws, T **p, uint64_t *cap, uint64_t want, uint64_t el
 
 // --------------------------------------------------------------- set prep ----
 
-// Mark one set: reject ids >= n and ids already marked (a repeat, or an id of R met
-// again in S: the sets must be disjoint), and set the membership bit of the internal
-// id.
-// set_bits marks internal ids, or original ids with by_orig.
-__global__ void k_mark_set(const uint32_t *__restrict__ ids, uint32_t cnt, uint32_t n,
-                           const uint32_t *__restrict__ perm, uint32_t *used_bits,
-                           uint32_t *set_bits, Control *ctl, bool by_orig) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
-        uint32_t id = ids[i];
+// Mark R and S: reject ids >= n and ids already marked (a repeat, or an id of R met again in
+// S: the sets must be disjoint), and set the members' bits -- S's by internal id, R's by
+// internal id or, with r_by_orig, by original id.
+__global__ void k_mark_sets(const uint32_t *__restrict__ R, uint32_t nR, const uint32_t *__restrict__ S, uint32_t nS,
+                            uint32_t n, const uint32_t *__restrict__ perm, uint32_t *used_bits, uint32_t *rbits,
+                            uint32_t *sbits, Control *ctl, bool r_by_orig) {
+    for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < uint64_t(nR) + nS; i += gridDim.x * blockDim.x) {
+        const bool in_r = i < nR;
+        const uint32_t id = in_r ? R[i] : S[i - nR];
         if (id >= n) {
             atomicOr(&ctl->err, 1u);
             continue;
         }
-        uint32_t bit = 1u << (id & 31);
-        uint32_t old = atomicOr(&used_bits[id >> 5], bit);
-        if (old & bit) {
+        const uint32_t bit = 1u << (id & 31);
+        if (atomicOr(&used_bits[id >> 5], bit) & bit) {
             atomicOr(&ctl->err, 2u);
             continue;
         }
-        const uint32_t in = by_orig ? id : perm[id];
-        atomicOr(&set_bits[in >> 5], 1u << (in & 31));
+        const uint32_t in = in_r && r_by_orig ? id : perm[id];
+        atomicOr(&(in_r ? rbits : sbits)[in >> 5], 1u << (in & 31));
     }
 }
 
@@ -482,14 +493,33 @@ __global__ void k_bits_count(const uint32_t *__restrict__ bits, uint32_t nwords,
     }
 }
 
-// Write the ids of the set bits in increasing order (R sorted by internal id, so a
-// tile holds R nodes of one neighbourhood).  The last block stores the total.
+// Write the ids of the set bits in increasing order, each through `map` when there is one
+// (R sorted by internal id, so a tile holds R nodes of one neighbourhood; or R in increasing
+// original id, written as internal ids).  The last block stores the total.  With no
+// block_sums a block counts the bits before it itself: cheaper than a launch of
+// k_bits_count while there are few blocks (up to COMPACT_BLOCKS).
+constexpr uint32_t COMPACT_BLOCKS = 16;
 __global__ void k_bits_compact(const uint32_t *__restrict__ bits, uint32_t nwords,
                                const uint32_t *__restrict__ block_sums, uint32_t nblocks,
-                               uint32_t *out, Control *ctl) {
+                               uint32_t *out, Control *ctl, const uint32_t *__restrict__ map) {
     __shared__ uint32_t warp_sum[32];
-    __shared__ uint32_t s_base;
-    if (threadIdx.x < 32) {
+    __shared__ uint32_t s_base, s_own;
+    if (!block_sums) {
+        uint32_t before = 0, own = 0;
+#pragma unroll 4
+        for (uint32_t j = threadIdx.x; j < blockIdx.x * 1024; j += 1024) before += __popc(bits[j]);
+        if (blockIdx.x * 1024 + threadIdx.x < nwords) own = __popc(bits[blockIdx.x * 1024 + threadIdx.x]);
+        if (threadIdx.x == 0) s_base = s_own = 0;
+        __syncthreads();
+        before = __reduce_add_sync(FULL, before);
+        own = __reduce_add_sync(FULL, own);
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&s_base, before);
+            atomicAdd(&s_own, own);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && blockIdx.x == nblocks - 1) ctl->r_count = s_base + s_own;
+    } else if (threadIdx.x < 32) {
         uint32_t s = 0;
         for (uint32_t b = threadIdx.x; b < blockIdx.x; b += 32) s += block_sums[b];
         s = __reduce_add_sync(FULL, s);
@@ -523,7 +553,8 @@ __global__ void k_bits_compact(const uint32_t *__restrict__ bits, uint32_t nword
     while (word) {
         uint32_t b = __ffs(word) - 1;
         word &= word - 1;
-        out[pos++] = i * 32 + b;
+        const uint32_t id = i * 32 + b;
+        out[pos++] = map ? map[id] : id;
     }
 }
 
@@ -1326,6 +1357,9 @@ constexpr uint32_t PG_ROW = 8;                  // arc slots per row
 constexpr uint64_t PG_ROWS_MAX = (uint64_t(1) << (32 - PG_BITS)) * 32 - 64;  // page ids fit beside the slot
 constexpr uint32_t PG_MAX = 1536;               // most pages of one group (196 KB of distances)
 __host__ __device__ constexpr int pg_groups(int W) { return W == 1 ? 4 : 1; }
+// a group's counters: sums, then maxima (Control::tel)
+enum { W_SCANS, W_ARCS, W_SLOT_ARCS, W_ROUNDS, W_BOUNDS, W_SLOTS, W_CYC_ROUND, W_CYC_BOUND, W_CYC_EMIT, W_N };
+enum { M_BALL, M_SEG, M_PAGES, M_N };
 // control words of a group, behind its queues
 enum {
     PC_PAGES, PC_CNT0, PC_CNT1, PC_CNT2, PC_MIN0, PC_MIN1, PC_FAIL, PC_ITEM, PC_BOUND, PC_BASE_LO, PC_BASE_HI, PC_FILL,
@@ -1456,8 +1490,6 @@ __global__ void __launch_bounds__(32 * W * pg_groups(W), W == 1 ? 8 : 32 / W) k_
     for (uint32_t i = gt; i < a.pg_buckets / 2; i += NT)
         reinterpret_cast<uint4 *>(table)[i] = make_uint4(PG_NONE, PG_NONE, PG_NONE, PG_NONE);
     // telemetry: counted per source in registers, added to the group's totals when it ends
-    enum { W_SCANS, W_ARCS, W_SLOT_ARCS, W_ROUNDS, W_BOUNDS, W_SLOTS, W_PAGES, W_CYC_ROUND, W_CYC_BOUND, W_CYC_EMIT, W_N };
-    enum { M_BALL, M_SEG, M_PAGES, M_N };
     __shared__ unsigned long long s_tel[G][W_N];
     __shared__ uint32_t s_max[G][M_N];
     __shared__ uint32_t s_wcnt[W];
@@ -1470,12 +1502,22 @@ __global__ void __launch_bounds__(32 * W * pg_groups(W), W == 1 ? 8 : 32 / W) k_
     const uint32_t nitems = a.range_list ? a.ntiles : nR1;
     const bool kcp = a.kcp_hist != nullptr;
     uint32_t t_mark = uint32_t(clock());
+    // W = 1: while many sources are left, a group draws its next one as it begins one, so
+    // that the counter's answer is there when it ends (towards the end it draws when it is
+    // free: a source drawn early would wait for its group while others idle)
+    uint32_t ahead = PG_NONE;
+    const uint32_t early = 2 * gridDim.x * G < nitems ? nitems - 2 * gridDim.x * G : 0;
 
     for (;;) {
-        uint32_t item = 0;
+        uint32_t item = ahead;
         if (W == 1) {
-            if (lane == 0) item = atomicAdd(&a.ctl->tile_next, 1u);
+            if (ahead == PG_NONE && lane == 0) item = atomicAdd(&a.ctl->tile_next, 1u);
             item = __shfl_sync(FULL, item, 0);
+            ahead = PG_NONE;
+            if (item < early) {
+                ahead = 0;  // (lane 0's alone is read)
+                if (lane == 0) ahead = atomicAdd(&a.ctl->tile_next, 1u);
+            }
         } else {
             if (gt == 0) ctl[PC_ITEM] = atomicAdd(&a.ctl->tile_next, 1u);
             __syncthreads();
@@ -1883,7 +1925,6 @@ __global__ void __launch_bounds__(32 * W * pg_groups(W), W == 1 ? 8 : 32 / W) k_
         if (gt == 0) {
             if (!fail) {
                 tel[W_SLOTS] += ball;
-                tel[W_PAGES] += pages;
                 s_max[grp][M_BALL] = max(s_max[grp][M_BALL], ball);
                 s_max[grp][M_SEG] = max(s_max[grp][M_SEG], total);
                 s_max[grp][M_PAGES] = max(s_max[grp][M_PAGES], pages);
@@ -1902,26 +1943,16 @@ __global__ void __launch_bounds__(32 * W * pg_groups(W), W == 1 ? 8 : 32 / W) k_
         t_mark = t_end;
         group_sync<W>();
     }
-    group_sync<W>();
-    if (gt == 0) {
-        const unsigned long long *tel = s_tel[grp];
-        atomicAdd(&a.ctl->scans, tel[W_SCANS]);
-        atomicAdd(&a.ctl->dirty_groups, tel[W_SCANS]);
-        atomicAdd(&a.ctl->round_items, tel[W_SCANS]);
-        atomicAdd(&a.ctl->round_arcs, tel[W_ARCS]);
-        atomicAdd(&a.ctl->slot_arcs, tel[W_SLOT_ARCS]);
-        atomicAdd(&a.ctl->slots, tel[W_SLOTS]);
-        atomicAdd(&a.ctl->slot_lanes, tel[W_SLOTS]);
-        atomicAdd(&a.ctl->pages, tel[W_PAGES]);
-        atomicAdd(&a.ctl->rounds, tel[W_ROUNDS]);
-        atomicAdd(&a.ctl->boundaries, tel[W_BOUNDS]);
-        atomicAdd(&a.ctl->cyc_round, tel[W_CYC_ROUND]);
-        atomicAdd(&a.ctl->cyc_bound, tel[W_CYC_BOUND]);
-        atomicAdd(&a.ctl->cyc_emit, tel[W_CYC_EMIT]);
-        atomicMax(&a.ctl->max_fill, s_max[grp][M_BALL]);
-        atomicMax(&a.ctl->src_max_ball, s_max[grp][M_BALL]);
-        atomicMax(&a.ctl->src_max_pages, s_max[grp][M_PAGES]);
-        atomicMax(&a.ctl->max_seg, s_max[grp][M_SEG]);
+    __syncthreads();
+    // the block's sums to its copy of the counters, in the order of Control's additions
+    if (threadIdx.x < W_N) {
+        unsigned long long t = 0;
+        for (uint32_t g = 0; g < G; g++) t += s_tel[g][threadIdx.x];
+        if (t) atomicAdd(&a.ctl->tel[blockIdx.x % 16][threadIdx.x], t);
+    } else if (threadIdx.x < W_N + M_N) {
+        uint32_t m = 0;
+        for (uint32_t g = 0; g < G; g++) m = max(m, s_max[g][threadIdx.x - W_N]);
+        if (m) atomicMax(&a.ctl->tel[blockIdx.x % 16][threadIdx.x], (unsigned long long)m);
     }
 }
 
@@ -2881,10 +2912,6 @@ __global__ void __launch_bounds__(W * 32, (3 * 8192) / MS) k_hash_coop(SearchArg
 // sorted by (u, v)) needs a scan of the counts and one placement pass, in which a warp
 // sorts one segment of up to 256 pairs in registers (bitonic network) and writes it.
 
-__global__ void k_seg_counts(const uint2 *__restrict__ seg, uint32_t n, uint32_t *cnt) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) cnt[i] = seg[i].y;
-}
-
 // Ascending bitonic sort of the warp's 32 E values, element lane * E + e in x[e].
 template <int E>
 __device__ __forceinline__ void warp_bitonic(unsigned long long (&x)[E], uint32_t lane) {
@@ -2954,21 +2981,95 @@ __device__ __forceinline__ void place_segment(uint32_t lane, uint32_t base, uint
     }
 }
 
-// One warp per source: its segment, sorted by v, at its offset off[si] of the result
-// (u, v, d arrays; or, when out_key is given, (key, d) records).
-__global__ void k_place(const uint2 *__restrict__ seg, const uint32_t *__restrict__ off, uint32_t n,
+constexpr uint32_t PLACE_MAX = 256;  // longest segment k_place sorts
+constexpr uint32_t PLACE_SEGS = 64;  // segments of one block, eight for each of its warps
+
+// Every source's segment, sorted by v, at its offset of the result (u, v, d arrays; or, when
+// out_key is given, (key, d) records).  The offsets are the running sum of the segments'
+// counts, found in the same launch: a block sums its own, publishes the sum, and adds up the
+// published sums of the blocks before it (state: epoch, kind -- 1 a block's own sum, 2 the sum
+// up to it --, count).  Blocks are numbered in the order they start, so the ones waited for
+// run or have ended; a wait is cut after about a second and reported as a failed check.
+// check_first: leave everything to the host unless the search completed and its pairs fit.
+__global__ void __launch_bounds__(256) k_place(const uint2 *__restrict__ seg, uint32_t n,
                         const unsigned long long *__restrict__ key, const uint32_t *__restrict__ val, uint32_t vbits,
-                        uint32_t umask, uint32_t *out_u, uint32_t *out_v, uint32_t *out_d,
-                        unsigned long long *out_key = nullptr, uint32_t *out_val = nullptr) {
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t warps = gridDim.x * (blockDim.x / 32);
+                        uint32_t umask, uint32_t *out_u, uint32_t *out_v, uint32_t *out_d, unsigned long long *out_key,
+                        uint32_t *out_val, uint64_t cap, unsigned long long *state, uint32_t epoch, Control *ctl,
+                        bool check_first) {
+    __shared__ uint32_t s_block, s_ok, s_base, s_off[PLACE_SEGS], s_half;
+    __shared__ uint2 s_seg[PLACE_SEGS];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (warp == 0) {
+        bool ok = true;
+        if (check_first) {
+            const uint32_t longest = lane < 16 ? uint32_t(__ldcg(&ctl->tel[lane][W_N + M_SEG])) : __ldcg(&ctl->max_seg);
+            ok = longest <= PLACE_MAX && !__ldcg(&ctl->err) && !__ldcg(&ctl->check[0]) && !__ldcg(&ctl->n_failed) &&
+                 __ldcg(&ctl->pairs) <= cap;
+        }
+        ok = __all_sync(FULL, ok);
+        if (lane == 0) {
+            s_ok = ok;
+            s_block = ok ? atomicAdd(&ctl->place_next, 1u) : 0u;
+        }
+    }
+    __syncthreads();
+    if (!s_ok) return;
+    const uint32_t b = s_block, first = b * PLACE_SEGS;
+    if (tid < PLACE_SEGS) {
+        const uint2 g = first + tid < n ? seg[first + tid] : make_uint2(0, 0);
+        s_seg[tid] = g;
+        uint32_t incl = g.y;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(FULL, incl, o);
+            if (lane >= uint32_t(o)) incl += t;
+        }
+        s_off[tid] = incl - g.y;
+        if (tid == 31) s_half = incl;
+        if (tid == PLACE_SEGS - 1) s_base = incl;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned long long tag = (unsigned long long)epoch << 34;
+        const uint32_t own = s_half + s_base;
+        if (lane == 0) atomicExch(&state[b], tag | (b ? 1ull : 2ull) << 32 | own);
+        uint32_t before = 0, tries = 0;
+        bool lost = false;
+        for (int32_t at = int32_t(b) - 1; at >= 0 && !lost;) {
+            const int32_t i = at - int32_t(lane);
+            unsigned long long w = tag | 2ull << 32;  // (before the first block: nothing)
+            for (;;) {
+                if (i >= 0) w = *(volatile unsigned long long *)&state[i];
+                const bool ready = (w >> 34) == epoch && ((w >> 32) & 3) != 0;
+                if (__all_sync(FULL, ready)) break;
+                if (++tries > 4000000u) {
+                    lost = true;
+                    break;
+                }
+            }
+            if (lost) break;
+            const uint32_t whole = __ballot_sync(FULL, ((w >> 32) & 3) == 2);
+            const uint32_t last = whole ? __ffs(whole) - 1 : 31;  // the nearest sum up to a block, or all own sums
+            before += __reduce_add_sync(FULL, lane <= last ? uint32_t(w) : 0u);
+            if (whole) break;
+            at -= 32;
+        }
+        if (lane == 0) {
+            if (b) atomicExch(&state[b], tag | 2ull << 32 | (before + own));
+            if (lost) record_check(ctl, 31, b, before);
+            s_base = before;
+            s_ok = !lost;
+        }
+    }
+    __syncthreads();
+    if (!s_ok) return;
     const unsigned long long vmask = (1ull << vbits) - 1;
-    for (uint32_t si = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); si < n; si += warps) {
-        const uint2 sg = seg[si];
+    for (uint32_t i = warp; i < PLACE_SEGS; i += 8) {
+        const uint2 sg = s_seg[i];
         const uint32_t cnt = sg.y;
         if (!cnt) continue;
         const uint32_t u = uint32_t(key[sg.x] >> vbits) & umask;
-        const uint32_t o = off[si];
+        const uint32_t o = s_base + s_off[i] + (i >= 32 ? s_half : 0u);
         if (cnt <= 32) place_segment<1>(lane, sg.x, cnt, o, u, key, val, vmask, out_u, out_v, out_d, out_key, out_val);
         else if (cnt <= 64) place_segment<2>(lane, sg.x, cnt, o, u, key, val, vmask, out_u, out_v, out_d, out_key, out_val);
         else if (cnt <= 128) place_segment<4>(lane, sg.x, cnt, o, u, key, val, vmask, out_u, out_v, out_d, out_key, out_val);
@@ -2976,14 +3077,6 @@ __global__ void k_place(const uint2 *__restrict__ seg, const uint32_t *__restric
     }
 }
 
-// Replace the original ids of list[0, min(cap, r_count)) by internal ids.
-__global__ void k_to_internal(uint32_t *list, uint32_t cap, const uint32_t *__restrict__ perm,
-                              const Control *__restrict__ ctl) {
-    const uint32_t n = min(cap, ctl->r_count);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) list[i] = perm[list[i]];
-}
-
-constexpr uint32_t PLACE_MAX = 256;  // longest segment k_place sorts
 
 // ------------------------------------------------------------- radix sort ----
 // LSD radix sort of (64-bit key, 32-bit value) records, 8 bits per pass.  Stable within
@@ -3293,7 +3386,26 @@ static void search(uint32_t T, Shape shape, const SearchArgs &a, uint32_t grid, 
 static Control read_control(Workspace *ws, cudaStream_t st) {
     RN_CUDA(cudaMemcpyAsync(ws->ctl_host, ws->ctl, sizeof(Control), cudaMemcpyDeviceToHost, st));
     RN_CUDA(cudaStreamSynchronize(st));
-    return *ws->ctl_host;
+    Control c = *ws->ctl_host;
+    for (const auto &t : c.tel) {
+        c.scans += t[W_SCANS];
+        c.dirty_groups += t[W_SCANS];
+        c.round_items += t[W_SCANS];
+        c.round_arcs += t[W_ARCS];
+        c.slot_arcs += t[W_SLOT_ARCS];
+        c.slots += t[W_SLOTS];
+        c.slot_lanes += t[W_SLOTS];
+        c.rounds += t[W_ROUNDS];
+        c.boundaries += t[W_BOUNDS];
+        c.cyc_round += t[W_CYC_ROUND];
+        c.cyc_bound += t[W_CYC_BOUND];
+        c.cyc_emit += t[W_CYC_EMIT];
+        c.max_fill = std::max(c.max_fill, uint32_t(t[W_N + M_BALL]));
+        c.src_max_ball = std::max(c.src_max_ball, uint32_t(t[W_N + M_BALL]));
+        c.max_seg = std::max(c.max_seg, uint32_t(t[W_N + M_SEG]));
+        c.src_max_pages = std::max(c.src_max_pages, uint32_t(t[W_N + M_PAGES]));
+    }
+    return c;
 }
 
 // Slots of the first map of a search: 8192 (narrow blocks, shared memory), 16384 (wide
@@ -3731,7 +3843,7 @@ static PageShape page_shape(uint32_t cap, uint32_t items, int sms, bool hier) {
     p.cap = cap;
     p.buckets = 32;
     while (p.buckets < 2 * cap && p.buckets < 2048) p.buckets *= 2;
-    p.queue = std::min<uint32_t>(std::max<uint32_t>(4 * cap, 64), 2048);
+    p.queue = std::min<uint32_t>(std::max<uint32_t>(2 * cap, 64), 2048);
     p.words = (32 * cap + 2 * p.buckets + cap + p.queue + PC_WORDS + 3) / 4 * 4;
     const uint32_t want = std::max<uint32_t>(1, (items + sms - 1) / sms);  // sources per SM
     const uint32_t most = cap <= 32 ? 2 : cap <= 100 ? 4 : cap <= 300 ? 8 : cap <= 700 ? 16 : 32;
@@ -3893,7 +4005,7 @@ static uint32_t source_first_map(const DeviceGraph &g, const Workspace *ws, uint
         // few more; with no history, the estimated ball at half-full pages, else 96 pages (a
         // join's first search, which its measured balls then size)
         const double seen = pages_at(ws, theta);
-        return page_cap(g, seen > 0 ? seen * 1.06 + 2 : first > 0 ? first / 16 + 16 : 96);
+        return page_cap(g, std::max(16.0, seen > 0 ? seen * 1.06 + 2 : first > 0 ? first / 16 + 16 : 96));
     }
     if (b <= 0) {
         if (first <= 0) return 2048;
@@ -3918,7 +4030,8 @@ static uint32_t source_first_map(const DeviceGraph &g, const Workspace *ws, uint
 // the next query's choice of path and map.
 static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs a, uint32_t nsrc, uint32_t ms0,
                                  uint32_t T, uint32_t theta, const std::vector<uint32_t> &inst_first,
-                                 cudaStream_t st, uint64_t *retried, bool learn_balls = true) {
+                                 cudaStream_t st, uint64_t *retried, bool learn_balls = true,
+                                 const std::function<void()> &after = {}) {
     a.n_nodes = g.n;
     a.n_arcs = g.arcs;
     a.range_list = nullptr;
@@ -3932,9 +4045,11 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
     const bool paged = by_pages(g, theta);
     if (nsrc) source_launch(g, paged, ms0, a, nsrc, ws, st);
     RN_CUDA(cudaEventRecord(ws->evs1, st));
+    if (after) after();  // work that needs no word from the host (it looks at the outcome itself)
     Control c = read_control(ws, st);
     ws->retry_ms = 0;
     ws->src_tiles = false;
+    ws->src_clean = !c.n_failed && !c.err && !c.check[0];
     ws->blocks_per_sm = !nsrc ? 0 : paged ? int(page_shape(ms0, nsrc, ws->num_sms, false).blocks) : source_blocks_per_sm(ms0);
     double ball = c.src_max_ball, pages = c.src_max_pages;
     // mean ball of the sources the first pass completed (0 when none did)
@@ -4047,15 +4162,15 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
     return c;
 }
 
-// Per-source segments of the warp search for nsrc sources, cleared on the stream.
-static uint2 *ensure_segments(Workspace *ws, uint32_t nsrc, cudaStream_t st) {
+// Per-source segments of the source search for nsrc sources (it writes every one, or reports
+// the source as failed).
+static uint2 *ensure_segments(Workspace *ws, uint32_t nsrc) {
     if (!ws->seg || ws->seg_cap < nsrc) {
         device_free(ws->seg);
         ws->seg = nullptr;
         ws->seg_cap = std::max<uint32_t>(nsrc, 1024);
         ws->seg = (uint2 *)device_alloc(size_t(ws->seg_cap) * 8);
     }
-    if (nsrc) RN_CUDA(cudaMemsetAsync(ws->seg, 0, size_t(nsrc) * 8, st));
     return ws->seg;
 }
 
@@ -4065,21 +4180,40 @@ static bool can_place(const Workspace *ws, const Control &c) {
     return !ws->src_tiles && c.max_seg <= PLACE_MAX && c.pairs <= ws->pair_cap && c.pairs < 0xFFFFFFFFull;
 }
 
-// The canonical order by placement: offsets from the segments' counts (source order is
-// the output order), then one warp per segment; with no `out`, into the workspace's
-// (keyA, valA) records instead, in (u, v) order.
-static void place_pairs(Workspace *ws, uint32_t nsrc, uint32_t vbits, uint32_t umask, rn_dpairs *out,
-                        cudaStream_t st) {
+static void check_control(const Control &c);
+
+// The canonical order by placement (k_place: source order is the output order): into `out`
+// or, with none, into the workspace's other (key, distance) records, in (u, v) order.  Before
+// the search's outcome is known (`early`) the kernel looks at it itself.
+static void place_launch(Workspace *ws, uint32_t nsrc, uint32_t vbits, uint32_t umask, rn_dpairs *out, uint64_t out_cap,
+                         cudaStream_t st, bool early) {
     if (!nsrc) return;
-    grow(ws, &ws->hist, &ws->hist_cap, hist_words(nsrc), 4);
-    const uint32_t nb = std::min<uint32_t>((nsrc + 255) / 256, 4096);
-    k_seg_counts<<<nb, 256, 0, st>>>(ws->seg, nsrc, ws->hist);
-    ws->launches += 1 + scan_hist(ws->hist, nsrc, st);
-    k_place<<<std::min<uint32_t>((nsrc + 7) / 8, 8192), 256, 0, st>>>(
-        ws->seg, ws->hist, nsrc, ws->keyA, ws->valA, vbits, umask, out ? out->u : nullptr, out ? out->v : nullptr,
-        out ? out->d : nullptr, out ? nullptr : ws->keyB, out ? nullptr : ws->valB);
+    const uint32_t nb = (nsrc + PLACE_SEGS - 1) / PLACE_SEGS;
+    if (ws->place_cap < nb) {
+        device_free(ws->place_state);
+        ws->place_state = nullptr;
+        ws->place_cap = std::max<uint32_t>(nb, 1024);
+        ws->place_state = (unsigned long long *)device_alloc(size_t(ws->place_cap) * 8);
+        RN_CUDA(cudaMemsetAsync(ws->place_state, 0, size_t(ws->place_cap) * 8, st));
+        ws->place_epoch = 0;
+    }
+    if (!early) RN_CUDA(cudaMemsetAsync(&ws->ctl->place_next, 0, 4, st));
+    ws->place_epoch = (ws->place_epoch + 1) & 0x3FFFFFFFu;
+    if (!ws->place_epoch) {  // (the epochs start again: no word of theirs may be left)
+        RN_CUDA(cudaMemsetAsync(ws->place_state, 0, size_t(ws->place_cap) * 8, st));
+        ws->place_epoch = 1;
+    }
+    k_place<<<nb, 256, 0, st>>>(ws->seg, nsrc, ws->keyA, ws->valA, vbits, umask, out ? out->u : nullptr,
+                                out ? out->v : nullptr, out ? out->d : nullptr, out ? nullptr : ws->keyB,
+                                out ? nullptr : ws->valB, std::min(ws->pair_cap, out_cap), ws->place_state, ws->place_epoch,
+                                ws->ctl, early);
     ws->launches++;
     RN_CUDA(cudaGetLastError());
+}
+
+static void place_pairs(Workspace *ws, uint32_t nsrc, uint32_t vbits, uint32_t umask, rn_dpairs *out, cudaStream_t st) {
+    place_launch(ws, nsrc, vbits, umask, out, out ? out->cap : ws->pair_cap, st, false);
+    check_control(read_control(ws, st));
     if (!out) {  // the placed records become the radix sort's input
         std::swap(ws->keyA, ws->keyB);
         std::swap(ws->valA, ws->valB);
@@ -4159,31 +4293,35 @@ void workspace_reserve(Workspace *ws, uint32_t max_r, uint64_t max_pairs) {
     }
 }
 
+static uint32_t mark_sets(const uint32_t *dR, uint32_t nR, const uint32_t *dS, uint32_t nS, const DeviceGraph &g,
+                          uint32_t *used, uint32_t *rbits, uint32_t *sbits, Control *ctl, bool by_orig, cudaStream_t st) {
+    const uint64_t ids = uint64_t(nR) + nS;
+    if (!ids) return 0;
+    k_mark_sets<<<uint32_t(std::min<uint64_t>((ids + 255) / 256, 4096)), 256, 0, st>>>(dR, nR, dS, nS, g.n, g.perm, used, rbits,
+                                                                                    sbits, ctl, by_orig);
+    return 1;
+}
+
+static uint32_t compact_bits(const uint32_t *bits, uint32_t nwords, uint32_t *block_sums, uint32_t *out, Control *ctl,
+                             const uint32_t *map, cudaStream_t st) {
+    const uint32_t nblocks = (nwords + 1023) / 1024;
+    const bool counted = nblocks > COMPACT_BLOCKS;
+    if (counted) k_bits_count<<<nblocks, 1024, 0, st>>>(bits, nwords, block_sums);
+    k_bits_compact<<<std::max<uint32_t>(nblocks, 1), 1024, 0, st>>>(bits, nwords, counted ? block_sums : nullptr,
+                                                                    std::max<uint32_t>(nblocks, 1), out, ctl, map);
+    return counted ? 2 : 1;
+}
+
 // a2: validate R and S on the device, build the S membership bitmap and the list of R
 // nodes in increasing internal id (so consecutive sources are graph neighbours).
 // by_orig: R in increasing original id instead (each source alone, so the order of
 // sources need not follow the graph; it is the output order).
 static void prep_sets(const DeviceGraph &g, Workspace *ws, const uint32_t *dR, uint32_t nR,
                       const uint32_t *dS, uint32_t nS, cudaStream_t st, bool by_orig = false) {
-    RN_CUDA(cudaMemsetAsync(ws->used_bits, 0, size_t(ws->nwords) * 4, st));
-    RN_CUDA(cudaMemsetAsync(ws->rbits, 0, size_t(ws->nwords) * 4, st));
-    RN_CUDA(cudaMemsetAsync(ws->sbits, 0, size_t(ws->nwords) * 4, st));
-    RN_CUDA(cudaMemsetAsync(ws->ctl, 0, sizeof(Control), st));
-    if (nR)
-        k_mark_set<<<std::min<uint32_t>((nR + 255) / 256, 4096), 256, 0, st>>>(dR, nR, g.n, g.perm, ws->used_bits,
-                                                                               ws->rbits, ws->ctl, by_orig);
-    if (nS)
-        k_mark_set<<<std::min<uint32_t>((nS + 255) / 256, 4096), 256, 0, st>>>(dS, nS, g.n, g.perm, ws->used_bits,
-                                                                               ws->sbits, ws->ctl, false);
+    RN_CUDA(cudaMemsetAsync(ws->ctl, 0, ws->clear_bytes, st));  // the control block and the three bitmaps
+    ws->launches += mark_sets(dR, nR, dS, nS, g, ws->used_bits, ws->rbits, ws->sbits, ws->ctl, by_orig, st);
     ensure_u32(&ws->rsorted, &ws->rsorted_cap, std::max<uint32_t>(nR, 1));
-    const uint32_t nblocks = (ws->nwords + 1023) / 1024;
-    k_bits_count<<<nblocks, 1024, 0, st>>>(ws->rbits, ws->nwords, ws->block_sums);
-    k_bits_compact<<<nblocks, 1024, 0, st>>>(ws->rbits, ws->nwords, ws->block_sums, nblocks, ws->rsorted, ws->ctl);
-    ws->launches += (nR ? 1 : 0) + (nS ? 1 : 0) + 2;
-    if (by_orig && nR) {
-        k_to_internal<<<std::min<uint32_t>((nR + 255) / 256, 4096), 256, 0, st>>>(ws->rsorted, nR, g.perm, ws->ctl);
-        ws->launches++;
-    }
+    ws->launches += compact_bits(ws->rbits, ws->nwords, ws->block_sums, ws->rsorted, ws->ctl, by_orig ? g.perm : nullptr, st);
     RN_CUDA(cudaGetLastError());
 }
 
@@ -4271,12 +4409,21 @@ void run_join(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint
     a.out_key = ws->keyA;
     a.out_d = ws->valA;
     a.out_cap = ws->pair_cap;
-    a.seg = place ? ensure_segments(ws, nR, st) : nullptr;
+    a.seg = place ? ensure_segments(ws, nR) : nullptr;
     a.swap_uv = from_s;
     uint64_t retried = 0;
     const std::vector<uint32_t> one_query;
+    // the placement is launched behind the search without waiting for its outcome, when the
+    // caller's buffers are there: the host learns of both together
+    bool early = false;
+    const std::function<void()> place_early = [&] {
+        if (!place || !nR || !out->u) return;
+        place_launch(ws, nR, vbits, 0xFFFFFFFFu, out, out->cap, st, true);
+        RN_CUDA(cudaEventRecord(ws->ev1, st));
+        early = true;
+    };
     auto search_pass = [&] {
-        return by_source ? source_search_all(g, ws, a, nR, ms0, T, theta, one_query, st, &retried)
+        return by_source ? source_search_all(g, ws, a, nR, ms0, T, theta, one_query, st, &retried, true, place_early)
                          : search_all(g, ws, T, a, ntiles, st, &retried, cfg.map_slots);
     };
     Control c;
@@ -4293,7 +4440,8 @@ void run_join(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint
         a.out_key = ws->keyA;
         a.out_d = ws->valA;
         a.out_cap = ws->pair_cap;
-        a.seg = place ? ensure_segments(ws, nR, st) : nullptr;
+        a.seg = place ? ensure_segments(ws, nR) : nullptr;
+        early = false;
         c = search_pass();
         check_control(c);
         if (c.pairs > ws->pair_cap) fail(RN_EINTERNAL, "pair count changed between passes");
@@ -4303,16 +4451,18 @@ void run_join(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint
     // a5: canonical order by (u, v), written straight into the caller's buffers: by
     // placing the warp search's per-source segments, else by a radix sort of all pairs
     Range rsort("rn.sort");
-    dpairs_reserve(out, np);
-    if (place && can_place(ws, c)) {
-        place_pairs(ws, nR, vbits, 0xFFFFFFFFu, out, st);
-    } else {
-        std::vector<int> shifts;
-        for (uint32_t sh = 0; sh < 2 * vbits; sh += 8) shifts.push_back(int(sh));
-        radix_sort_to_pairs(ws, np, shifts, vbits, out, st);
+    if (!(early && ws->src_clean && can_place(ws, c) && np <= out->cap)) {
+        dpairs_reserve(out, np);
+        if (place && can_place(ws, c)) {
+            place_pairs(ws, nR, vbits, 0xFFFFFFFFu, out, st);
+        } else {
+            std::vector<int> shifts;
+            for (uint32_t sh = 0; sh < 2 * vbits; sh += 8) shifts.push_back(int(sh));
+            radix_sort_to_pairs(ws, np, shifts, vbits, out, st);
+        }
+        RN_CUDA(cudaEventRecord(ws->ev1, st));
     }
     out->n = np;
-    RN_CUDA(cudaEventRecord(ws->ev1, st));
     RN_CUDA(cudaEventSynchronize(ws->ev1));
     float ms = 0, sms = 0;
     RN_CUDA(cudaEventElapsedTime(&ms, ws->ev0, ws->ev1));
@@ -4509,10 +4659,18 @@ void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg
     a.inst_swap = any_swap ? ws->mq_swap : nullptr;
     stats->from_s = any_swap;
     const bool place = by_source && g.iperm_inverts_perm && !any_swap;
-    a.seg = place ? ensure_segments(ws, total, st) : nullptr;
+    a.seg = place ? ensure_segments(ws, total) : nullptr;
     uint64_t retried = 0;
+    const uint32_t umask = vbits >= 32 ? 0xFFFFFFFFu : (1u << vbits) - 1;
+    bool early = false;
+    std::vector<unsigned long long> cnt(nq);
+    const std::function<void()> place_early = [&] {  // as for one join
+        if (!place || !total || !out->u) return;
+        place_launch(ws, total, vbits, umask, out, out->cap, st, true);
+        early = true;
+    };
     auto search_pass = [&] {
-        return by_source ? source_search_all(g, ws, a, total, ms0, T, max_bound, first, st, &retried)
+        return by_source ? source_search_all(g, ws, a, total, ms0, T, max_bound, first, st, &retried, true, place_early)
                          : search_all(g, ws, T, a, 0, st, &retried, cfg.map_slots, true, &ranges);
     };
     Control c = search_pass();
@@ -4525,12 +4683,12 @@ void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg
         a.out_key = ws->keyA;
         a.out_d = ws->valA;
         a.out_cap = ws->pair_cap;
-        a.seg = place ? ensure_segments(ws, total, st) : nullptr;
+        a.seg = place ? ensure_segments(ws, total) : nullptr;
+        early = false;
         c = search_pass();
         check_control(c);
         if (c.pairs > ws->pair_cap) fail(RN_EINTERNAL, "pair count changed between passes");
     }
-    std::vector<unsigned long long> cnt(nq);
     RN_CUDA(cudaMemcpyAsync(cnt.data(), ws->mq_counts, size_t(nq) * 8, cudaMemcpyDeviceToHost, st));
     RN_CUDA(cudaStreamSynchronize(st));
     counts->assign(cnt.begin(), cnt.end());
@@ -4539,9 +4697,9 @@ void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg
     if (sum != c.pairs) fail(RN_EINTERNAL, "per-query pair counts do not add up");
     const uint64_t np = c.pairs;
     Range rsort("rn.sort");
-    dpairs_reserve(out, np);
-    const uint32_t umask = vbits >= 32 ? 0xFFFFFFFFu : (1u << vbits) - 1;
-    if (place && can_place(ws, c)) {
+    if (early && ws->src_clean && can_place(ws, c) && np <= out->cap) {
+        // placed already
+    } else if (dpairs_reserve(out, np); place && can_place(ws, c)) {
         place_pairs(ws, total, vbits, umask, out, st);  // sources in (query, u) order
     } else {
         std::vector<int> shifts;
@@ -4646,7 +4804,6 @@ void run_join_noalloc(const DeviceGraph &g, uint32_t median_w, const uint32_t *d
     uint32_t *hist = base + NA_HIST;
     uint32_t *slab = base + NA_SLAB;
     const uint32_t nwords = (g.n + 31) / 32;
-    const uint32_t nblocks = (nwords + 1023) / 1024;
 
     // the array keeps the previous call's contents: clear what must start at zero, and
     // put the slab rows back to INF (a previous call may have stopped half-way)
@@ -4655,12 +4812,8 @@ void run_join_noalloc(const DeviceGraph &g, uint32_t median_w, const uint32_t *d
     RN_CUDA(cudaMemsetAsync(rbits, 0, size_t(nwords) * 4, st));
     RN_CUDA(cudaMemsetAsync(sbits, 0, size_t(nwords) * 4, st));
     RN_CUDA(cudaMemsetAsync(slab, 0xFF, size_t(NA_BLOCKS) * SMEM_H * 32 * 4, st));
-    if (nR)
-        k_mark_set<<<std::min<uint32_t>((nR + 255) / 256, 4096), 256, 0, st>>>(dR, nR, g.n, g.perm, used_bits, rbits, ctl, false);
-    if (nS)
-        k_mark_set<<<std::min<uint32_t>((nS + 255) / 256, 4096), 256, 0, st>>>(dS, nS, g.n, g.perm, used_bits, sbits, ctl, false);
-    k_bits_count<<<nblocks, 1024, 0, st>>>(rbits, nwords, bsums);
-    k_bits_compact<<<nblocks, 1024, 0, st>>>(rbits, nwords, bsums, nblocks, rsorted, ctl);
+    mark_sets(dR, nR, dS, nS, g, used_bits, rbits, sbits, ctl, false, st);
+    compact_bits(rbits, nwords, bsums, rsorted, ctl, nullptr, st);
     RN_CUDA(cudaGetLastError());
 
     constexpr uint32_t T = 32;
@@ -4884,11 +5037,12 @@ void run_kcp(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint3
     a.kcp_k = k;
     a.swap_uv = from_s;
     // a source's ball at the k-th distance holds about (k / |R|) (n / |S|) nodes (each
-    // source's share of the k pairs, one S node per n / |S| nodes): a warp's map passes at
+    // source's share of the k pairs, one S node per n / |S| nodes): a hashed map's passes at
     // bucket boundaries and emission do not pay for balls of a few dozen nodes, which the
-    // tile search shares between the sources of a tile
+    // tile search shares between the sources of a tile (the search by pages visits the ball's
+    // pages alone and takes them all)
     const double kth_ball = nR && nS ? double(k) / nR * (double(g.n) / nS) : 0.0;
-    const bool warp_ok = cfg.tile_width == 1 || kth_ball >= 64.0;
+    const bool hashed_ok = cfg.tile_width == 1 || kth_ball >= 64.0;
     // the first radius: where about 1.25 k pairs are expected, the balls growing as the
     // workspace's last warp search measured them (mean ball at its bound, times the
     // squared radius ratio) or, with none behind it, as a lattice's 2 (r / w_med)^2; a
@@ -4906,17 +5060,23 @@ void run_kcp(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint3
     uint32_t passes = 0;
     Control c{};
     unsigned long long scans = 0;
-    bool any_tiles = false, last_by_source = false;
+    bool any_tiles = false, last_by_source = false, early = false;
+    const std::function<void()> place_early = [&] {  // as for a join, into records
+        if (!last_by_source || !nR) return;
+        place_launch(ws, nR, vbits, 0xFFFFFFFFu, nullptr, ws->pair_cap, st, true);
+        early = true;
+    };
     for (;;) {
         // every pass takes the warp search while the balls at tau fit a warp map
-        const bool by_source = warp_ok && use_source_search(g, ws, cfg, uint32_t(tau), median_w);
+        const bool by_source = (hashed_ok || by_pages(g, uint32_t(tau))) && use_source_search(g, ws, cfg, uint32_t(tau), median_w);
         const uint32_t delta = choose_delta(cfg, median_w, by_source);
         // the warp search takes R in output order and records each source's segment
         const bool place = by_source && g.iperm_inverts_perm && !from_s;
         prep_sets(g, ws, dR, nR, dS, nS, st, place);
         a.src = ws->rsorted;  // prep_sets may have (re)allocated the R list
-        a.seg = place ? ensure_segments(ws, nR, st) : nullptr;
+        a.seg = place ? ensure_segments(ws, nR) : nullptr;
         last_by_source = place;
+        early = false;
         RN_CUDA(cudaMemsetAsync(hist, 0, KCP_BINS * 4, st));
         k_set_u32<<<1, 1, 0, st>>>(theta_live, uint32_t(tau));
         ws->launches++;
@@ -4933,7 +5093,7 @@ void run_kcp(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint3
             c = source_search_all(g, ws, a, nR,
                                   source_first_map(g, ws, uint32_t(tau), first_ball_estimate(g, uint32_t(tau), median_w)), T,
                                   uint32_t(tau), {}, st,
-                                  &retried, false);
+                                  &retried, false, place_early);
         } else {
             a.tile_src = tile_src;
             c = search_all(g, ws, T, a, ntiles, st, &retried, cfg.map_slots);
@@ -4963,7 +5123,12 @@ void run_kcp(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint3
         // the warp search's segments placed in (u, v) order, then a stable LSD sort of all
         // candidates by distance alone: (d, u, v) order, of which the first k are the answer
         // (no selection: three distance passes instead of the (u, v) digits' six)
-        place_pairs(ws, nR, vbits, 0xFFFFFFFFu, nullptr, st);
+        if (early && ws->src_clean) {
+            std::swap(ws->keyA, ws->keyB);
+            std::swap(ws->valA, ws->valB);
+        } else {
+            place_pairs(ws, nR, vbits, 0xFFFFFFFFu, nullptr, st);
+        }
         dpairs_reserve(out, m);
         std::vector<int> shifts;
         const uint32_t dbits = bits_for(uint32_t(std::min<uint64_t>(tau, RN_THETA_MAX)) + 1);

@@ -76,6 +76,9 @@ bool pinned_give(void *p) {
 }
 }  // namespace
 
+// Results of up to this many pairs are written to the host by a kernel, larger ones copied.
+constexpr uint64_t TO_HOST_MAX = uint64_t(1) << 20;
+
 void to_host_pairs(const rn_dpairs &d, rn_pairs *out, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
     out->n = d.n;
@@ -95,9 +98,13 @@ void to_host_pairs(const rn_dpairs &d, rn_pairs *out, void *stream) {
         }
     }
     if (d.n) {
-        cudaMemcpyAsync(out->u, d.u, d.n * 4, cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(out->v, d.v, d.n * 4, cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(out->d, d.d, d.n * 4, cudaMemcpyDeviceToHost, st);
+        if (blk && d.n <= TO_HOST_MAX) {
+            triple_to_host(d.u, d.v, d.d, d.n, blk, stream);
+        } else {
+            cudaMemcpyAsync(out->u, d.u, d.n * 4, cudaMemcpyDeviceToHost, st);
+            cudaMemcpyAsync(out->v, d.v, d.n * 4, cudaMemcpyDeviceToHost, st);
+            cudaMemcpyAsync(out->d, d.d, d.n * 4, cudaMemcpyDeviceToHost, st);
+        }
         cudaError_t e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) {
             rn_pairs_free(out);

@@ -128,6 +128,23 @@ void copy_to_device(void *dst, const void *src, size_t bytes, void *stream) {
     RN_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, (cudaStream_t)stream));
 }
 
+// Three device arrays of n words to dst, dst + n and dst + 2 n in page-locked host memory, which
+// the kernel writes itself: one launch instead of three copies and their gaps.
+__global__ void k_to_host(const uint32_t *__restrict__ u, const uint32_t *__restrict__ v, const uint32_t *__restrict__ d,
+                          uint64_t n, uint32_t *dst) {
+    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += uint64_t(gridDim.x) * blockDim.x) {
+        const uint32_t a = u[i], b = v[i], c = d[i];
+        dst[i] = a;
+        dst[n + i] = b;
+        dst[2 * n + i] = c;
+    }
+}
+
+void triple_to_host(const uint32_t *u, const uint32_t *v, const uint32_t *d, uint64_t n, uint32_t *dst, void *stream) {
+    if (n) k_to_host<<<uint32_t(std::min<uint64_t>((n + 255) / 256, 1216)), 256, 0, (cudaStream_t)stream>>>(u, v, d, n, dst);
+    RN_CUDA(cudaGetLastError());
+}
+
 void stream_sync(void *stream) { RN_CUDA(cudaStreamSynchronize((cudaStream_t)stream)); }
 
 void dpairs_reserve(rn_dpairs *p, uint64_t cap) {
@@ -230,6 +247,7 @@ struct Control {
     uint32_t err;          // 1: id >= n, 2: repeated id or R/S overlap
     uint32_t r_count;      // R nodes after validation
     uint32_t place_next;   // blocks of the placement started
+    uint32_t max_rank;     // most pairs of one u (searches from S)
     uint32_t tile_next;    // work-queue head of the persistent search
     uint32_t n_failed;     // tiles whose slab overflowed
     unsigned long long pairs;
@@ -319,6 +337,7 @@ struct Workspace {
     uint64_t pair_cap = 0;
     uint32_t *hist = nullptr;
     size_t hist_cap = 0;
+    uint32_t *ranks = nullptr;  // searches from S: the marked ids before every word of used_bits
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, evs0 = nullptr, evs1 = nullptr;
     DeviceShared *own_sh = nullptr;  // a slab of its own (workspace_set_slab), else null
     cudaEvent_t evr = nullptr;  // end of the last retry launch
@@ -414,6 +433,7 @@ void workspace_destroy(Workspace *ws) {
     device_free(ws->own_gmap);
     device_free(ws->seg);
     device_free(ws->place_state);
+    device_free(ws->ranks);
     device_free(ws->slist);
     if (ws->own_sh) {
         device_free(ws->own_sh->gretry);
@@ -1332,7 +1352,7 @@ __global__ void __launch_bounds__(THREADS, (THREADS == NARROW ? CTAS_PER_SM : 1)
 // no CSR offset is read first; a node with more arcs goes on in a row of its own behind an
 // arc of weight 0), then issues the four table lookups, the four atomicMin and the pushes.
 // When the queue drains, a pass over the ball's pages takes the least pending distance and
-// collects the next bucket.  W = 1: four groups per block, lanes synchronise with
+// collects the next bucket.  W = 1: two groups per block, lanes synchronise with
 // __syncwarp.  W > 1: one group per block, one barrier per round: a scan takes its item's
 // dirty bit with an atomicAnd, so scans and relaxations of a round need no barrier between
 // them (a distance improved before the scan is read by it; one improved after it makes the
@@ -1356,7 +1376,7 @@ constexpr uint32_t PG_BOUND_MAX = 0x7FFFFFFEu;  // 2 d + 1 stays below PG_CLEAN
 constexpr uint32_t PG_ROW = 8;                  // arc slots per row
 constexpr uint64_t PG_ROWS_MAX = (uint64_t(1) << (32 - PG_BITS)) * 32 - 64;  // page ids fit beside the slot
 constexpr uint32_t PG_MAX = 1536;               // most pages of one group (196 KB of distances)
-__host__ __device__ constexpr int pg_groups(int W) { return W == 1 ? 4 : 1; }
+__host__ __device__ constexpr int pg_groups(int W) { return W == 1 ? 2 : 1; }
 // a group's counters: sums, then maxima (Control::tel)
 enum { W_SCANS, W_ARCS, W_SLOT_ARCS, W_ROUNDS, W_BOUNDS, W_SLOTS, W_CYC_ROUND, W_CYC_BOUND, W_CYC_EMIT, W_N };
 enum { M_BALL, M_SEG, M_PAGES, M_N };
@@ -1471,7 +1491,7 @@ __device__ __forceinline__ uint32_t page_slot(uint32_t *table, uint32_t *pkey, u
 }
 
 template <int W, bool HIER>
-__global__ void __launch_bounds__(32 * W * pg_groups(W), W == 1 ? 8 : 32 / W) k_source_search(SearchArgs a) {
+__global__ void __launch_bounds__(32 * W * pg_groups(W), 32 / (W * pg_groups(W))) k_source_search(SearchArgs a) {
     constexpr uint32_t NT = 32 * W;
     constexpr int G = pg_groups(W);
     extern __shared__ __align__(16) uint32_t smem[];
@@ -2913,8 +2933,8 @@ __global__ void __launch_bounds__(W * 32, (3 * 8192) / MS) k_hash_coop(SearchArg
 // sorts one segment of up to 256 pairs in registers (bitonic network) and writes it.
 
 // Ascending bitonic sort of the warp's 32 E values, element lane * E + e in x[e].
-template <int E>
-__device__ __forceinline__ void warp_bitonic(unsigned long long (&x)[E], uint32_t lane) {
+template <int E, class T>
+__device__ __forceinline__ void warp_bitonic(T (&x)[E], uint32_t lane) {
 #pragma unroll
     for (uint32_t k = 2; k <= 32u * E; k <<= 1) {
 #pragma unroll
@@ -2924,7 +2944,7 @@ __device__ __forceinline__ void warp_bitonic(unsigned long long (&x)[E], uint32_
                 const bool lower = (lane & lj) == 0;
 #pragma unroll
                 for (int e = 0; e < E; e++) {
-                    const unsigned long long p = __shfl_xor_sync(FULL, x[e], lj);
+                    const T p = __shfl_xor_sync(FULL, x[e], lj);
                     const bool up = ((lane * E + e) & k) == 0;
                     x[e] = (lower == up) ? (x[e] < p ? x[e] : p) : (x[e] < p ? p : x[e]);
                 }
@@ -2933,7 +2953,7 @@ __device__ __forceinline__ void warp_bitonic(unsigned long long (&x)[E], uint32_
                 for (int e = 0; e < E; e++) {
                     if ((e & j) == 0) {
                         const bool up = ((lane * E + e) & k) == 0;
-                        const unsigned long long lo = x[e], hi = x[e ^ j];
+                        const T lo = x[e], hi = x[e ^ j];
                         if ((lo > hi) == up) {
                             x[e] = hi;
                             x[e ^ j] = lo;
@@ -2952,12 +2972,27 @@ __device__ __forceinline__ void place_segment(uint32_t lane, uint32_t base, uint
                                               uint32_t *out_u, uint32_t *out_v, uint32_t *out_d,
                                               unsigned long long *out_key, uint32_t *out_val) {
     unsigned long long x[E];
+    if (vmask < 1ull << 24) {
+        // v and the pair's place in the segment in one word: a third of the instructions of
+        // sorting (v, d), whose d is fetched afterwards
+        uint32_t w[E];
 #pragma unroll
-    for (int e = 0; e < E; e++) {
-        const uint32_t i = lane * E + e;
-        x[e] = i < cnt ? ((key[base + i] & vmask) << 32) | val[base + i] : ~0ull;  // v, then d
+        for (int e = 0; e < E; e++) {
+            const uint32_t i = lane * E + e;
+            w[e] = i < cnt ? uint32_t(key[base + i] & vmask) << 8 | i : 0xFFFFFFFFu;
+        }
+        warp_bitonic<E>(w, lane);
+#pragma unroll
+        for (int e = 0; e < E; e++)
+            x[e] = (unsigned long long)(w[e] >> 8) << 32 | (lane * E + e < cnt ? val[base + (w[e] & 255)] : 0u);
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; e++) {
+            const uint32_t i = lane * E + e;
+            x[e] = i < cnt ? ((key[base + i] & vmask) << 32) | val[base + i] : ~0ull;  // v, then d
+        }
+        warp_bitonic<E>(x, lane);
     }
-    warp_bitonic<E>(x, lane);
     if (out_key) {  // records (key, distance) for a sort that follows
         const unsigned long long khi = key[base] & ~vmask;
 #pragma unroll
@@ -3077,6 +3112,105 @@ __global__ void __launch_bounds__(256) k_place(const uint2 *__restrict__ seg, ui
     }
 }
 
+
+// ---- searches from S: the pairs of one u lie in many segments (one per source v), so they
+// are counted per u -- by its rank among the marked ids, which order as the ids do --, moved
+// to their u's place and sorted by v there.  Five to seven launches over the pairs instead of a
+// radix sort's three to five for every eight bits of (u, v).
+
+// Set bits before every word (of an id's bitmap: the id's rank is this plus the bits before it
+// in its word).  With no block_sums a block counts the words before it itself.
+__global__ void k_word_ranks(const uint32_t *__restrict__ bits, uint32_t nwords, const uint32_t *__restrict__ block_sums,
+                             uint32_t *out) {
+    __shared__ uint32_t warp_sum[32], s_base;
+    if (threadIdx.x == 0) s_base = 0;
+    __syncthreads();
+    uint32_t before = 0;
+    if (block_sums) {
+        for (uint32_t b = threadIdx.x; b < blockIdx.x; b += 1024) before += block_sums[b];
+    } else {
+#pragma unroll 4
+        for (uint32_t j = threadIdx.x; j < blockIdx.x * 1024; j += 1024) before += __popc(bits[j]);
+    }
+    before = __reduce_add_sync(FULL, before);
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 1024 + threadIdx.x;
+    if (lane == 0 && before) atomicAdd(&s_base, before);
+    const uint32_t c = i < nwords ? __popc(bits[i]) : 0;
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= uint32_t(o)) incl += t;
+    }
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();
+    uint32_t base = s_base;
+    for (uint32_t w = 0; w < warp; w++) base += warp_sum[w];
+    if (i < nwords) out[i] = base + incl - c;
+}
+
+__device__ __forceinline__ uint32_t rank_of(const uint32_t *__restrict__ bits, const uint32_t *__restrict__ ranks, uint32_t id) {
+    return ranks[id >> 5] + __popc(bits[id >> 5] & ((1u << (id & 31)) - 1));
+}
+
+// Each pair's place among those of its u, and the pairs of every u; the most of one u goes to
+// the control block.  The number of pairs is read on the device (cap of them at most).
+__global__ void k_rank_count(const unsigned long long *__restrict__ key, uint64_t cap, uint32_t vbits,
+                             const uint32_t *__restrict__ bits, const uint32_t *__restrict__ ranks, uint32_t *count,
+                             uint32_t *place, Control *ctl) {
+    const uint64_t n = min((unsigned long long)cap, __ldcg(&ctl->pairs));
+    uint32_t most = 0;
+    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += uint64_t(gridDim.x) * blockDim.x) {
+        const uint32_t at = atomicAdd(&count[rank_of(bits, ranks, uint32_t(key[i] >> vbits))], 1u);
+        place[i] = at;
+        most = max(most, at + 1);
+    }
+    most = __reduce_max_sync(FULL, most);
+    if ((threadIdx.x & 31) == 0 && most) atomicMax(&ctl->max_rank, most);
+}
+
+// The pairs at their u's places (start[rank] on): u in the result, (v, d) as one word.
+__global__ void k_rank_scatter(const unsigned long long *__restrict__ key, const uint32_t *__restrict__ d, uint64_t n,
+                               uint32_t vbits, const uint32_t *__restrict__ bits, const uint32_t *__restrict__ ranks,
+                               const uint32_t *__restrict__ start, const uint32_t *__restrict__ place, uint32_t *out_u,
+                               unsigned long long *vd) {
+    const unsigned long long vmask = (1ull << vbits) - 1;
+    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += uint64_t(gridDim.x) * blockDim.x) {
+        const unsigned long long k = key[i];
+        const uint32_t u = uint32_t(k >> vbits), at = start[rank_of(bits, ranks, u)] + place[i];
+        out_u[at] = u;
+        vd[at] = (k & vmask) << 32 | d[i];
+    }
+}
+
+template <int E>
+__device__ __forceinline__ void rank_segment(uint32_t lane, uint32_t at, uint32_t cnt, const unsigned long long *__restrict__ vd,
+                                             uint32_t *out_v, uint32_t *out_d) {
+    unsigned long long x[E];
+#pragma unroll
+    for (int e = 0; e < E; e++) x[e] = lane * E + e < cnt ? vd[at + lane * E + e] : ~0ull;
+    warp_bitonic<E>(x, lane);
+#pragma unroll
+    for (int e = 0; e < E; e++)
+        if (lane * E + e < cnt) {
+            out_v[at + lane * E + e] = uint32_t(x[e] >> 32);
+            out_d[at + lane * E + e] = uint32_t(x[e]);
+        }
+}
+
+// One warp per rank: its pairs (up to PLACE_MAX) by v.
+__global__ void k_rank_place(const uint32_t *__restrict__ start, uint32_t n, uint64_t pairs,
+                             const unsigned long long *__restrict__ vd, uint32_t *out_v, uint32_t *out_d) {
+    const uint32_t lane = threadIdx.x & 31, warps = gridDim.x * (blockDim.x / 32);
+    for (uint32_t r = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); r < n; r += warps) {
+        const uint32_t at = start[r], cnt = (r + 1 < n ? start[r + 1] : uint32_t(pairs)) - at;
+        if (!cnt) continue;
+        if (cnt <= 32) rank_segment<1>(lane, at, cnt, vd, out_v, out_d);
+        else if (cnt <= 64) rank_segment<2>(lane, at, cnt, vd, out_v, out_d);
+        else if (cnt <= 128) rank_segment<4>(lane, at, cnt, vd, out_v, out_d);
+        else rank_segment<8>(lane, at, cnt, vd, out_v, out_d);
+    }
+}
 
 // ------------------------------------------------------------- radix sort ----
 // LSD radix sort of (64-bit key, 32-bit value) records, 8 bits per pass.  Stable within
@@ -3267,16 +3401,260 @@ __global__ void k_rs_scatter(const unsigned long long *__restrict__ kin, const u
     }
 }
 
+// A kernel's attributes (its dynamic shared-memory limit, the carveout) belong to the
+// device that was current when they were set, so every kernel sets them once per device.
+constexpr int MAX_DEVICES = 64;
+static int attr_device() {
+    int d = 0;
+    RN_CUDA(cudaGetDevice(&d));
+    if (d < 0 || d >= MAX_DEVICES) fail(RN_EINVAL, "device ordinal out of range");
+    return d;
+}
+
+// ---- large sorts: one launch per digit
+// The three-kernel pass above reads the records twice, scans a histogram per block and digit
+// with three more launches and scatters records one by one.  From SWEEP_MIN records on, one
+// kernel counts every digit of the sort at once, and a pass is a single launch: a block ranks
+// its 4096 records, publishes its count per digit, adds up the counts of the blocks before it
+// (each digit looks back on its own thread until a block whose running sum is known), orders
+// its records in shared memory and writes runs of equal digits.  Blocks take their number in
+// the order they start, so the ones looked back at run or have ended; a wait is cut after
+// about a second and reported as a failed check.
+constexpr uint64_t SWEEP_MIN = 1u << 18, SWEEP_FEW = 1u << 15;  // (SWEEP_FEW: from five passes on)
+constexpr uint64_t SWEEP_MAX = 1u << 30;  // counts leave two bits of their word for the kind
+constexpr int SWEEP_THREADS = 512, SWEEP_WARPS = SWEEP_THREADS / 32;
+constexpr int SWEEP_ROUNDS = 8;
+constexpr int SWEEP_LOOK = 8;
+constexpr uint32_t SWEEP_TILE = SWEEP_THREADS * SWEEP_ROUNDS;
+constexpr uint32_t SWEEP_PASSES = 12;
+constexpr uint32_t SWEEP_HEAD = SWEEP_PASSES * 256 + 64;  // digit counts, then the passes' block counters
+constexpr size_t SWEEP_SMEM = size_t(SWEEP_TILE) * 12 + SWEEP_WARPS * 256 * 4;
+
+struct SweepShifts {
+    int n, shift[SWEEP_PASSES];
+};
+
+__global__ void __launch_bounds__(256) k_sweep_count(const unsigned long long *__restrict__ keys,
+                                                     const uint32_t *__restrict__ vals, uint64_t n, SweepShifts sh,
+                                                     uint32_t *counts) {
+    __shared__ uint32_t cnt[SWEEP_PASSES][256];
+    for (int p = 0; p < sh.n; p++) cnt[p][threadIdx.x] = 0;
+    __syncthreads();
+    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += uint64_t(gridDim.x) * blockDim.x) {
+        const unsigned long long k = keys[i];
+        const uint32_t v = vals[i];
+#pragma unroll
+        for (int p = 0; p < int(SWEEP_PASSES); p++)
+            if (p < sh.n) atomicAdd(&cnt[p][rs_digit(k, v, sh.shift[p])], 1u);
+    }
+    __syncthreads();
+    for (int p = 0; p < sh.n; p++)
+        if (cnt[p][threadIdx.x]) atomicAdd(&counts[p * 256 + threadIdx.x], cnt[p][threadIdx.x]);
+}
+
+// state: per block and digit its count (kind 1) or the running sum up to it (kind 2), the
+// kind in the top two bits; zero before the sort.
+__global__ void __launch_bounds__(SWEEP_THREADS, 2) k_sweep(const unsigned long long *__restrict__ kin,
+                                                      const uint32_t *__restrict__ vin, unsigned long long *kout,
+                                                      uint32_t *vout, uint64_t n, int shift,
+                                                      const uint32_t *__restrict__ counts, uint32_t *ticket,
+                                                      uint32_t *state, uint32_t *out_u, uint32_t *out_v, uint32_t *out_d,
+                                                      uint32_t vbits, uint32_t umask, Control *ctl) {
+    extern __shared__ __align__(16) uint32_t sweep_smem[];
+    unsigned long long *const skey = reinterpret_cast<unsigned long long *>(sweep_smem);
+    uint32_t *const sval = sweep_smem + 2 * SWEEP_TILE;
+    uint32_t(*const wcnt)[256] = reinterpret_cast<uint32_t(*)[256]>(sval + SWEEP_TILE);
+    __shared__ uint32_t s_block, s_scan[8], s_scan2[8], s_base[256], s_lost;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lt = (1u << lane) - 1;
+    if (tid == 0) {
+        s_block = atomicAdd(ticket, 1u);
+        s_lost = 0;
+    }
+    for (uint32_t i = tid; i < SWEEP_WARPS * 256; i += SWEEP_THREADS) wcnt[0][i] = 0;
+    __syncthreads();
+    const uint32_t block = s_block;
+    const uint64_t first = uint64_t(block) * SWEEP_TILE + uint64_t(warp) * (SWEEP_ROUNDS * 32);
+    unsigned long long k[SWEEP_ROUNDS];
+    uint32_t v[SWEEP_ROUNDS], rank[SWEEP_ROUNDS];
+#pragma unroll
+    for (int r = 0; r < SWEEP_ROUNDS; r++) {
+        const uint64_t i = first + uint64_t(r) * 32 + lane;
+        k[r] = i < n ? kin[i] : 0ull;
+        v[r] = i < n ? vin[i] : 0u;
+    }
+#pragma unroll
+    for (int r = 0; r < SWEEP_ROUNDS; r++) {
+        const bool valid = first + uint64_t(r) * 32 + lane < n;
+        const uint32_t d = rs_digit(k[r], v[r], shift);
+        uint32_t peers = __ballot_sync(FULL, valid);  // the lanes with this lane's digit
+#pragma unroll
+        for (int b = 0; b < 8; b++) {
+            const uint32_t m = __ballot_sync(FULL, (d >> b) & 1u);
+            peers &= (d >> b) & 1u ? m : ~m;
+        }
+        const uint32_t before = valid ? wcnt[warp][d] : 0u;
+        __syncwarp();
+        rank[r] = before + __popc(peers & lt);
+        if (valid && !(peers & lt)) wcnt[warp][d] = before + __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    // thread d of the first 256: the warps' offsets within digit d, the block's count, its start
+    // in the block's order, and the digit's start in the sorted records
+    const bool digit = tid < 256;
+    uint32_t own = 0, all = 0;
+    if (digit) {
+        for (int w = 0; w < SWEEP_WARPS; w++) {
+            const uint32_t c = wcnt[w][tid];
+            wcnt[w][tid] = own;
+            own += c;
+        }
+        all = counts[tid];
+        *(volatile uint32_t *)(state + size_t(block) * 256 + tid) = (block ? 1u : 2u) << 30 | own;
+    }
+    uint32_t x = own, y = all;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t a = __shfl_up_sync(FULL, x, o), b = __shfl_up_sync(FULL, y, o);
+        if (lane >= uint32_t(o)) {
+            x += a;
+            y += b;
+        }
+    }
+    if (digit && lane == 31) {
+        s_scan[warp] = x;
+        s_scan2[warp] = y;
+    }
+    __syncthreads();
+    if (digit) {
+        uint32_t local = x - own, global = y - all;
+        for (uint32_t w = 0; w < warp; w++) {
+            local += s_scan[w];
+            global += s_scan2[w];
+        }
+        uint32_t before = 0, tries = 0;
+        bool lost = false;
+        bool done = block == 0;
+        for (int64_t b = int64_t(block) - 1; !done && !lost; b -= SWEEP_LOOK) {
+            uint32_t s[SWEEP_LOOK];  // read together: one after another they cost an L2 trip each
+#pragma unroll
+            for (int j = 0; j < SWEEP_LOOK; j++)
+                s[j] = b - j >= 0 ? *(volatile uint32_t *)(state + size_t(b - j) * 256 + tid) : 2u << 30;
+#pragma unroll
+            for (int j = 0; j < SWEEP_LOOK; j++) {
+                if (done || lost) continue;
+                while (!(s[j] >> 30)) {
+                    if (++tries > 4000000u) {
+                        lost = true;
+                        break;
+                    }
+                    s[j] = *(volatile uint32_t *)(state + size_t(b - j) * 256 + tid);
+                }
+                before += s[j] & 0x3FFFFFFFu;
+                done = s[j] >> 31;
+            }
+        }
+        if (lost) {
+            record_check(ctl, 32, block, tid);
+            s_lost = 1;
+        } else if (block) {
+            *(volatile uint32_t *)(state + size_t(block) * 256 + tid) = 2u << 30 | (before + own);
+        }
+        for (int w = 0; w < SWEEP_WARPS; w++) wcnt[w][tid] += local;
+        s_base[tid] = global + before - local;  // (a record's place is this plus its place in the block)
+    }
+    __syncthreads();
+    if (s_lost) return;  // (nothing is written past the records)
+#pragma unroll
+    for (int r = 0; r < SWEEP_ROUNDS; r++) {
+        if (first + uint64_t(r) * 32 + lane < n) {
+            const uint32_t at = wcnt[warp][rs_digit(k[r], v[r], shift)] + rank[r];
+            skey[at] = k[r];
+            sval[at] = v[r];
+        }
+    }
+    __syncthreads();
+    const uint64_t left = n - uint64_t(block) * SWEEP_TILE;
+    const uint32_t count = left < SWEEP_TILE ? uint32_t(left) : SWEEP_TILE;
+    const unsigned long long vmask = (1ull << vbits) - 1;
+    for (uint32_t i = tid; i < count; i += SWEEP_THREADS) {
+        const unsigned long long key = skey[i];
+        const uint32_t val = sval[i], pos = s_base[rs_digit(key, val, shift)] + i;
+        if (out_u) {
+            out_u[pos] = uint32_t(key >> vbits) & umask;
+            out_v[pos] = uint32_t(key & vmask);
+            out_d[pos] = val;
+        } else {
+            kout[pos] = key;
+            vout[pos] = val;
+        }
+    }
+}
+
+// Words of `hist` a sort of n records needs.
+static uint64_t sort_words(uint64_t n) {
+    const uint64_t rs = hist_words((n + RS_TILE - 1) / RS_TILE * 256);
+    return n < SWEEP_FEW ? rs : std::max<uint64_t>(rs, SWEEP_HEAD + (n + SWEEP_TILE - 1) / SWEEP_TILE * 256 * SWEEP_PASSES);
+}
+
+static bool sweeps(uint64_t n, size_t passes) {
+    return (n >= SWEEP_MIN || (n >= SWEEP_FEW && passes >= 5)) && n < SWEEP_MAX && passes && passes <= SWEEP_PASSES;
+}
+
+// The sort of (k0, v0) by the listed digits in single-launch passes, with (k1, v1) as the other
+// buffers; the last pass writes the struct-of-arrays result when out_u is given.  Returns the
+// kernels launched.
+static uint32_t sweep_sort(unsigned long long *k0, uint32_t *v0, unsigned long long *k1, uint32_t *v1, uint64_t n,
+                           const std::vector<int> &shifts, uint32_t *hist, uint32_t *out_u, uint32_t *out_v, uint32_t *out_d,
+                           uint32_t vbits, uint32_t umask, Control *ctl, cudaStream_t st) {
+    static std::once_flag once[MAX_DEVICES];
+    std::call_once(once[attr_device()], [&] {
+        RN_CUDA(cudaFuncSetAttribute(k_sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SWEEP_SMEM)));
+    });
+    const uint32_t nb = uint32_t((n + SWEEP_TILE - 1) / SWEEP_TILE);
+    const uint32_t passes = uint32_t(shifts.size());
+    SweepShifts sh{};
+    sh.n = int(passes);
+    for (uint32_t p = 0; p < passes; p++) sh.shift[p] = shifts[p];
+    RN_CUDA(cudaMemsetAsync(hist, 0, (SWEEP_HEAD + size_t(nb) * 256 * passes) * 4, st));
+    k_sweep_count<<<std::min<uint32_t>(nb, 1024), 256, 0, st>>>(k0, v0, n, sh, hist);
+    for (uint32_t p = 0; p < passes; p++) {
+        const bool last = out_u && p + 1 == passes;
+        k_sweep<<<nb, SWEEP_THREADS, SWEEP_SMEM, st>>>(k0, v0, k1, v1, n, shifts[p], hist + p * 256,
+                                                    hist + SWEEP_PASSES * 256 + p, hist + SWEEP_HEAD + size_t(p) * nb * 256,
+                                                    last ? out_u : nullptr, last ? out_v : nullptr, last ? out_d : nullptr,
+                                                    vbits, umask, ctl);
+        std::swap(k0, k1);
+        std::swap(v0, v1);
+    }
+    RN_CUDA(cudaGetLastError());
+    return passes + 1;
+}
+
 // Sort n (key, value) records by the listed digit shifts (least significant first; a
 // shift >= 64 takes the value's bits), passing between (k0, v0) and (k1, v1); returns the
 // pair of buffers that holds the sorted records.
+static void check_control(const Control &c);
+
+// A sort's failed waits are reported in the control block: its check words are copied behind
+// the sort (queue_check) and looked at after the next synchronisation (late_check).
+static void queue_check(Workspace *ws, cudaStream_t st) {
+    RN_CUDA(cudaMemcpyAsync(ws->ctl_host->check, ws->ctl->check, sizeof(ws->ctl->check), cudaMemcpyDeviceToHost, st));
+}
+static void late_check(const Workspace *ws) { check_control(*ws->ctl_host); }
+
 static std::pair<unsigned long long *, uint32_t *> sort_kv(Workspace *ws, unsigned long long *k0, uint32_t *v0,
                                                            unsigned long long *k1, uint32_t *v1, uint64_t n,
                                                            const std::vector<int> &shifts, cudaStream_t st) {
     if (n == 0) return {k0, v0};
     if (n > 0xFFFFFFFFull) fail(RN_EINVAL, "more than 2^32 - 1 records to sort");
     const uint32_t nblocks = uint32_t((n + RS_TILE - 1) / RS_TILE);
-    grow(ws, &ws->hist, &ws->hist_cap, hist_words(uint64_t(nblocks) * 256), 4);
+    grow(ws, &ws->hist, &ws->hist_cap, sort_words(n), 4);
+    if (sweeps(n, shifts.size())) {
+        ws->launches += sweep_sort(k0, v0, k1, v1, n, shifts, ws->hist, nullptr, nullptr, nullptr, 32, 0, ws->ctl, st);
+        queue_check(ws, st);
+        return shifts.size() % 2 ? std::make_pair(k1, v1) : std::make_pair(k0, v0);
+    }
     for (int sh : shifts) {
         k_rs_hist<<<nblocks, RS_THREADS, 0, st>>>(k0, v0, n, sh, ws->hist, nblocks);
         ws->launches += scan_hist(ws->hist, nblocks * 256, st) + 2;
@@ -3296,7 +3674,13 @@ static void radix_sort_to_pairs(Workspace *ws, uint64_t n, const std::vector<int
     if (n == 0) return;
     if (n > 0xFFFFFFFFull) fail(RN_EINVAL, "more than 2^32 - 1 result pairs");
     const uint32_t nblocks = uint32_t((n + RS_TILE - 1) / RS_TILE);
-    grow(ws, &ws->hist, &ws->hist_cap, hist_words(uint64_t(nblocks) * 256), 4);
+    grow(ws, &ws->hist, &ws->hist_cap, sort_words(n), 4);
+    if (sweeps(n, shifts.size())) {
+        ws->launches += sweep_sort(ws->keyA, ws->valA, ws->keyB, ws->valB, n, shifts, ws->hist, out->u, out->v, out->d, vbits,
+                                   umask, ws->ctl, st);
+        queue_check(ws, st);
+        return;
+    }
     unsigned long long *ki = ws->keyA, *ko = ws->keyB;
     uint32_t *vi = ws->valA, *vo = ws->valB;
     for (size_t p = 0; p < shifts.size(); p++) {
@@ -3325,16 +3709,6 @@ static uint32_t bits_for(uint32_t n) {
 // lives in global memory, the two near queues and the staged items.
 static size_t search_smem(uint32_t H, bool gmap, int threads) {
     return (gmap ? 0 : size_t(H) * 12) + size_t(qcap_of(threads)) * 8 + size_t(icap_of(threads)) * 20;
-}
-
-// A kernel's attributes (its dynamic shared-memory limit, the carveout) belong to the
-// device that was current when they were set, so every kernel sets them once per device.
-constexpr int MAX_DEVICES = 64;
-static int attr_device() {
-    int d = 0;
-    RN_CUDA(cudaGetDevice(&d));
-    if (d < 0 || d >= MAX_DEVICES) fail(RN_EINVAL, "device ordinal out of range");
-    return d;
 }
 
 template <int L, bool GMAP, int THREADS>
@@ -3832,12 +4206,11 @@ struct PageShape {
 // displaced from its home bucket stops a step's 128 arc slots for a probe, and at one bucket a
 // page (1% of the pages displaced) that cost 2.06 ms against 1.70 with balls of 190 pages, 0.94
 // against 0.90 on the 264k-node join; four buckets a page cost an SM more groups than they
-// save.  The warps: one while the maps leave an SM sixteen
-// warps, since warps that share a ball wait for each other at every round, else the fewest
-// that give it 24, and never more than a round of the ball has items for.  Measured with
-// 1 / 2 / 4 / 8 / 16 warps, ms a call: 1.07M-node join (balls of up to 50 pages) 1.45 / 1.87 /
-// 2.35 / 3.57 / 6.6; 264k-node join (80 pages) 0.95 / 0.93 / 0.95 / 1.26 / 2.0; balls of up to
-// 190 pages 3.5 / 2.2 / 1.7 / 1.8 / 2.5, and 1.6 with eight where four warps make 16 of an SM.
+// save.  The warps: one while the maps leave an SM sixteen, since warps that share a ball wait
+// for each other at every round, else the fewest that give it 28, and never more than a round
+// of the ball has items for.  Measured with 1 / 2 / 4 / 8 / 16 warps, ms a call: 1.07M-node join
+// (balls of up to 50 pages) 1.45 / 1.87 / 2.35 / 3.57 / 6.6; 264k-node join (80 pages) - / 0.86 /
+// 0.89 / 1.20 / -; balls of up to 190 pages with 4 / 5 / 8 warps 1.49 / 1.42 / 1.58.
 static PageShape page_shape(uint32_t cap, uint32_t items, int sms, bool hier) {
     PageShape p{};
     p.cap = cap;
@@ -3847,13 +4220,13 @@ static PageShape page_shape(uint32_t cap, uint32_t items, int sms, bool hier) {
     p.words = (32 * cap + 2 * p.buckets + cap + p.queue + PC_WORDS + 3) / 4 * 4;
     const uint32_t want = std::max<uint32_t>(1, (items + sms - 1) / sms);  // sources per SM
     const uint32_t most = cap <= 32 ? 2 : cap <= 100 ? 4 : cap <= 300 ? 8 : cap <= 700 ? 16 : 32;
-    for (uint32_t W = 1;; W *= 2) {
+    for (uint32_t W : {1u, 2u, 4u, 5u, 8u, 16u, 32u}) {
         const uint32_t G = pg_groups(int(W));
         p.warps = W;
         p.smem = size_t(p.words) * 4 * G;
-        p.blocks = std::min<uint32_t>(uint32_t(233472 / (p.smem + 1024 + 640)), W == 1 ? 8 : 32 / W);
+        p.blocks = std::min<uint32_t>(uint32_t(233472 / (p.smem + 1024 + 256)), 32 / (W * G));
         p.groups = p.blocks * G;
-        if (hier ? (W == 4 || (W == 1 && cap <= 96)) : p.blocks && (W >= most || W * std::min(p.groups, want) >= (W == 1 ? 16u : 24u))) break;
+        if (hier ? (W == 4 || (W == 1 && cap <= 96)) : p.blocks && (W >= most || W * std::min(p.groups, want) >= (W == 1 ? 16u : 28u))) break;
     }
     if (!p.blocks) fail(RN_EINTERNAL, "a group's pages do not fit an SM");
     return p;
@@ -3892,6 +4265,7 @@ static void page_launch(const DeviceGraph &g, uint32_t cap, SearchArgs a, uint32
             case 1: launch_pages<1, false>(a, p, grid, st); break;
             case 2: launch_pages<2, false>(a, p, grid, st); break;
             case 4: launch_pages<4, false>(a, p, grid, st); break;
+            case 5: launch_pages<5, false>(a, p, grid, st); break;
             case 8: launch_pages<8, false>(a, p, grid, st); break;
             case 16: launch_pages<16, false>(a, p, grid, st); break;
             default: launch_pages<32, false>(a, p, grid, st); break;
@@ -4180,8 +4554,6 @@ static bool can_place(const Workspace *ws, const Control &c) {
     return !ws->src_tiles && c.max_seg <= PLACE_MAX && c.pairs <= ws->pair_cap && c.pairs < 0xFFFFFFFFull;
 }
 
-static void check_control(const Control &c);
-
 // The canonical order by placement (k_place: source order is the output order): into `out`
 // or, with none, into the workspace's other (key, distance) records, in (u, v) order.  Before
 // the search's outcome is known (`early`) the kernel looks at it itself.
@@ -4283,7 +4655,7 @@ void workspace_reserve(Workspace *ws, uint32_t max_r, uint64_t max_pairs) {
     ensure_ranges(&ws->failed, &ws->failed_cap, std::max<uint32_t>(max_r, 1));
     ensure_ranges(&ws->failed2, &ws->failed2_cap, std::max<uint32_t>(max_r, 1));
     ensure_pairs(ws, max_pairs);
-    grow(ws, &ws->hist, &ws->hist_cap, hist_words((max_pairs + RS_TILE - 1) / RS_TILE * 256), 4);
+    grow(ws, &ws->hist, &ws->hist_cap, sort_words(max_pairs), 4);
     ensure_slist(ws);
     if (!ws->seg || ws->seg_cap < max_r) {  // the warp search's per-source segments
         device_free(ws->seg);
@@ -4414,9 +4786,30 @@ void run_join(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint
     uint64_t retried = 0;
     const std::vector<uint32_t> one_query;
     // the placement is launched behind the search without waiting for its outcome, when the
-    // caller's buffers are there: the host learns of both together
+    // caller's buffers are there: the host learns of both together.  Searches from S: the
+    // count of every u's pairs
     bool early = false;
+    const bool by_rank = by_source && from_s && g.iperm_inverts_perm && uint64_t(nR) + nS < (1u << 30);
+    const uint32_t nranks = nR + nS;  // (ranks among all marked ids; S's have no pairs)
     const std::function<void()> place_early = [&] {
+        if (by_rank) {
+            if (!ws->ranks) {
+                ws->ranks = (uint32_t *)device_alloc(std::max<size_t>(ws->nwords, 1) * 4);
+                ws->bytes += size_t(ws->nwords) * 4;
+            }
+            grow(ws, &ws->hist, &ws->hist_cap, hist_words(nranks), 4);
+            const uint32_t nblocks = std::max<uint32_t>((ws->nwords + 1023) / 1024, 1);
+            const bool counted = nblocks > COMPACT_BLOCKS;
+            if (counted) k_bits_count<<<nblocks, 1024, 0, st>>>(ws->used_bits, ws->nwords, ws->block_sums);
+            k_word_ranks<<<nblocks, 1024, 0, st>>>(ws->used_bits, ws->nwords, counted ? ws->block_sums : nullptr, ws->ranks);
+            RN_CUDA(cudaMemsetAsync(ws->hist, 0, size_t(nranks) * 4, st));
+            k_rank_count<<<uint32_t(ws->num_sms) * 8, 256, 0, st>>>(ws->keyA, ws->pair_cap, vbits, ws->used_bits, ws->ranks,
+                                                                    ws->hist, ws->valB, ws->ctl);
+            RN_CUDA(cudaGetLastError());
+            ws->launches += counted ? 3 : 2;
+            early = true;
+            return;
+        }
         if (!place || !nR || !out->u) return;
         place_launch(ws, nR, vbits, 0xFFFFFFFFu, out, out->cap, st, true);
         RN_CUDA(cudaEventRecord(ws->ev1, st));
@@ -4451,9 +4844,16 @@ void run_join(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint
     // a5: canonical order by (u, v), written straight into the caller's buffers: by
     // placing the warp search's per-source segments, else by a radix sort of all pairs
     Range rsort("rn.sort");
-    if (!(early && ws->src_clean && can_place(ws, c) && np <= out->cap)) {
+    if (!(early && !by_rank && ws->src_clean && can_place(ws, c) && np <= out->cap)) {
         dpairs_reserve(out, np);
-        if (place && can_place(ws, c)) {
+        if (by_rank && early && ws->src_clean && np && c.max_rank <= PLACE_MAX && np < 0xFFFFFFFFull) {
+            ws->launches += scan_hist(ws->hist, nranks, st) + 2;
+            k_rank_scatter<<<uint32_t(std::min<uint64_t>((np + 255) / 256, 8192)), 256, 0, st>>>(
+                ws->keyA, ws->valA, np, vbits, ws->used_bits, ws->ranks, ws->hist, ws->valB, out->u, ws->keyB);
+            k_rank_place<<<std::min<uint32_t>((nranks + 7) / 8, 8192), 256, 0, st>>>(ws->hist, nranks, np, ws->keyB, out->v,
+                                                                                     out->d);
+            RN_CUDA(cudaGetLastError());
+        } else if (place && can_place(ws, c)) {
             place_pairs(ws, nR, vbits, 0xFFFFFFFFu, out, st);
         } else {
             std::vector<int> shifts;
@@ -4464,6 +4864,7 @@ void run_join(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint
     }
     out->n = np;
     RN_CUDA(cudaEventSynchronize(ws->ev1));
+    late_check(ws);
     float ms = 0, sms = 0;
     RN_CUDA(cudaEventElapsedTime(&ms, ws->ev0, ws->ev1));
     RN_CUDA(cudaEventElapsedTime(&sms, ws->evs0, ws->evs1));
@@ -4709,6 +5110,7 @@ void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg
     out->n = np;
     RN_CUDA(cudaEventRecord(ws->ev1, st));
     RN_CUDA(cudaEventSynchronize(ws->ev1));
+    late_check(ws);
     float ms = 0, sms = 0;
     RN_CUDA(cudaEventElapsedTime(&ms, ws->ev0, ws->ev1));
     RN_CUDA(cudaEventElapsedTime(&sms, ws->evs0, ws->evs1));
@@ -5173,6 +5575,7 @@ void run_kcp(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint3
     }
     RN_CUDA(cudaEventRecord(ws->ev1, st));
     RN_CUDA(cudaEventSynchronize(ws->ev1));
+    late_check(ws);
     float ms = 0, sms = 0;
     RN_CUDA(cudaEventElapsedTime(&ms, ws->ev0, ws->ev1));
     RN_CUDA(cudaEventElapsedTime(&sms, ws->evs0, ws->evs1));
@@ -5341,22 +5744,20 @@ static void points_graph(const DeviceGraph &g, const std::vector<uint32_t> &perm
     for (uint32_t i = 0; i < np; i++) {
         const uint4 f = found[key_of[i]];
         const rn_point &x = i < nR ? R[i] : S[i - nR];
-        const std::string who = (i < nR ? "R[" + std::to_string(i) : "S[" + std::to_string(i - nR)) + "]";
+        const auto who = [&] { return (i < nR ? "R[" + std::to_string(i) : "S[" + std::to_string(i - nR)) + "]"; };
         if (f.x == EMPTY || f.y == EMPTY || f.z != f.w)
-            fail(RN_EINVAL, who + ": {" + std::to_string(x.a) + ", " + std::to_string(x.b) + "} is not an undirected edge");
-        if (pts[i].pos_raw > f.z) fail(RN_EINVAL, who + ": t is longer than its edge");
+            fail(RN_EINVAL, who() + ": {" + std::to_string(x.a) + ", " + std::to_string(x.b) + "} is not an undirected edge");
+        if (pts[i].pos_raw > f.z) fail(RN_EINVAL, who() + ": t is longer than its edge");
         pos[i] = pts[i].from_p ? pts[i].pos_raw : f.z - pts[i].pos_raw;
     }
-    // node ids: R points in the order of their edges (locality), then S points
+    // node ids: the points in the order of their edges, R's and S's alike, so that the points a
+    // ball meets share pages (S's in the order given scattered them: 10,000 points on a 48k-node
+    // graph made the search by pages slower than the hashed one)
     std::vector<uint32_t> node(np), rank_ids(np);
-    {
-        uint32_t nextR = 0, nextS = 0;
-        for (uint32_t j = 0; j < np; j++) {
-            const uint32_t i = order[j];
-            if (i < nR) node[i] = g.n + nextR++;
-        }
-        for (uint32_t i = nR; i < np; i++) node[i] = g.n + nR + nextS++;
-        for (uint32_t i = 0; i < np; i++) rank_ids[node[i] - g.n] = i < nR ? i : i - nR;
+    for (uint32_t j = 0; j < np; j++) {
+        const uint32_t i = order[j];
+        node[i] = g.n + j;
+        rank_ids[j] = i < nR ? i : i - nR;
     }
     // chains: per edge, its points by position (then index), links between neighbours
     std::vector<uint32_t> tail(2 * size_t(np) * 2);  // object rows: (col, w) x 2 per point node
@@ -5448,7 +5849,7 @@ static void points_graph(const DeviceGraph &g, const std::vector<uint32_t> &perm
         ps->cap_ids = std::max<uint32_t>(np, 1024);
         ps->ids = (uint32_t *)device_alloc(size_t(ps->cap_ids) * 4);
     }
-    if (np) RN_CUDA(cudaMemcpyAsync(ps->ids, perm_tail.data(), size_t(np) * 4, cudaMemcpyHostToDevice, st));
+    if (np) RN_CUDA(cudaMemcpyAsync(ps->ids, node.data(), size_t(np) * 4, cudaMemcpyHostToDevice, st));
     RN_CUDA(cudaStreamSynchronize(st));  // the host vectors above are temporaries
 }
 
@@ -5625,6 +6026,7 @@ struct HierState {
     };
     std::map<std::string, Buf> bufs;
     unsigned long long *count = nullptr, *count_host = nullptr;  // 4 device counters, pinned copy
+    uint64_t candidates = 0;  // pairs and candidates of the last query: room for the next one's
     template <class T>
     T *get(const char *name, uint64_t n) {
         Buf &b = bufs[name];
@@ -5748,9 +6150,11 @@ __global__ void k_exit_compact(const unsigned long long *__restrict__ key, const
         const unsigned long long k = key[i];
         const uint32_t j = head_at[i] + head[i] - 1;
         if (head[i]) f_list[j] = uint32_t(k >> 32);
+        uint32_t least = d[i];  // (a run of equal keys, one or two long, is in no order of distance)
+        for (uint64_t r = i + 1; r < m && key[r] == k; r++) least = min(least, d[r]);
         e_key[keep_at[i]] = ((unsigned long long)j << 32) | uint32_t(k);
-        e_off[keep_at[i]] = d[i];
-        atomicMin(&fmin[j], d[i]);
+        e_off[keep_at[i]] = least;
+        atomicMin(&fmin[j], least);
     }
 }
 
@@ -5795,27 +6199,50 @@ __global__ void k_hier_combine(const unsigned long long *__restrict__ e_key, con
                                const uint32_t *__restrict__ hd, const uint32_t *__restrict__ src,
                                const uint32_t *__restrict__ iperm, uint32_t theta, uint32_t vbits,
                                unsigned long long *c_key, uint32_t *c_d, uint64_t cap, unsigned long long *count) {
-    const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1;
-    const uint64_t warps = uint64_t(gridDim.x) * (blockDim.x / 32);
+    // a block takes eight routes at a time, counts their candidates and draws their places with
+    // one addition to the counter (an addition per route was most of the time)
+    __shared__ uint32_t s_cnt[8];
+    __shared__ unsigned long long s_at;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lt = (1u << lane) - 1;
     const unsigned long long vmask = (1ull << vbits) - 1;
-    for (uint64_t i = uint64_t(blockIdx.x) * (blockDim.x / 32) + (threadIdx.x >> 5); i < ne; i += warps) {
-        const unsigned long long ek = e_key[i];
-        const uint32_t j = uint32_t(ek >> 32), si = uint32_t(ek), off = e_off[i];
-        const uint2 r = range[j];
-        const unsigned long long u = (unsigned long long)iperm[src[si]] << vbits;
-        for (uint32_t h0 = r.x; h0 < r.y; h0 += 32) {
-            const uint32_t h = h0 + lane;
-            const bool ok = h < r.y && uint64_t(off) + hd[h] <= theta;
-            const uint32_t b = __ballot_sync(FULL, ok);
-            if (!b) continue;
-            unsigned long long at = 0;
-            if (lane == 0) at = atomicAdd(count, (unsigned long long)__popc(b));
-            at = __shfl_sync(FULL, at, 0) + __popc(b & lt);
-            if (ok && at < cap) {
-                c_key[at] = u | (hkey[h] & vmask);
-                c_d[at] = off + hd[h];
+    for (uint64_t i0 = uint64_t(blockIdx.x) * 8; i0 < ne; i0 += uint64_t(gridDim.x) * 8) {
+        const uint64_t i = i0 + warp;
+        uint32_t off = 0, si = 0, n = 0;
+        uint2 r = make_uint2(0, 0);
+        if (i < ne) {
+            const unsigned long long ek = e_key[i];
+            si = uint32_t(ek);
+            off = e_off[i];
+            r = range[uint32_t(ek >> 32)];
+        }
+        for (uint32_t h = r.x + lane; h < r.y; h += 32) n += uint64_t(off) + hd[h] <= theta;
+        n = __reduce_add_sync(FULL, n);
+        if (lane == 0) s_cnt[warp] = n;
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < 8; w++) {
+            if (w < warp) before += s_cnt[w];
+            total += s_cnt[w];
+        }
+        if (threadIdx.x == 0 && total) s_at = atomicAdd(count, (unsigned long long)total);
+        __syncthreads();
+        if (n) {
+            unsigned long long at = s_at + before;
+            const unsigned long long u = (unsigned long long)iperm[src[si]] << vbits;
+            for (uint32_t h0 = r.x; h0 < r.y; h0 += 32) {
+                const uint32_t h = h0 + lane;
+                const bool ok = h < r.y && uint64_t(off) + hd[h] <= theta;
+                const uint32_t b = __ballot_sync(FULL, ok);
+                const unsigned long long to = at + __popc(b & lt);
+                if (ok && to < cap) {
+                    c_key[to] = u | (hkey[h] & vmask);
+                    c_d[to] = off + hd[h];
+                }
+                at += __popc(b);
             }
         }
+        __syncthreads();  // s_cnt and s_at are read before the next eight routes'
     }
 }
 
@@ -5831,8 +6258,11 @@ __global__ void k_first_compact(const unsigned long long *__restrict__ key, cons
                                 unsigned long long *okey, uint32_t *od) {
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < m; i += uint64_t(gridDim.x) * blockDim.x) {
         if (!first[i]) continue;
-        okey[at[i]] = key[i];
-        od[at[i]] = d[i];
+        const unsigned long long k = key[i];
+        uint32_t least = d[i];  // (a run of equal keys is in no order of distance)
+        for (uint64_t r = i + 1; r < m && key[r] == k; r++) least = min(least, d[r]);
+        okey[at[i]] = k;
+        od[at[i]] = least;
     }
 }
 
@@ -5965,7 +6395,6 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
     // The join within bound bnd: every pair's least distance, sorted by (u, v), as records
     // (orig(u) << vbits | orig(v), d) in (*ok, *od).
     auto join_at = [&](uint32_t bnd, unsigned long long **ok, uint32_t **od) -> uint64_t {
-        const int dbits = int(bits_for(uint32_t(std::min<uint64_t>(bnd + 1ull, 0xFFFFFFFFull))));
         // 1. local searches: pairs inside each source's part, routes to its border nodes
         mark();
         ensure_pairs(ws, std::max<uint64_t>(ws->pair_cap, uint64_t(nR) * 64));
@@ -6043,7 +6472,6 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
         unsigned long long *xk2 = h->get<unsigned long long>("ex_key2", nx);
         uint32_t *xd2 = h->get<uint32_t>("ex_d2", nx);
         std::vector<int> sh;
-        add_shifts(&sh, 0, uint32_t(dbits), 64);                      // offset
         add_shifts(&sh, 0, bits_for(std::max<uint32_t>(nR, 2)));      // si
         add_shifts(&sh, 32, 32 + vbits);                              // orig(f)
         const auto xs = sort_kv(ws, xk, xd, xk2, xd2, nx, sh, st);
@@ -6061,6 +6489,7 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
             RN_CUDA(cudaMemcpyAsync(&tot[0], keep_at + nx, 4, cudaMemcpyDeviceToHost, st));
             RN_CUDA(cudaMemcpyAsync(&tot[1], head_at + nx, 4, cudaMemcpyDeviceToHost, st));
             RN_CUDA(cudaStreamSynchronize(st));
+            late_check(ws);
             ne = tot[0];
             nf = tot[1];
         }
@@ -6132,7 +6561,7 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
         mark();
         // 4. candidates through the exit arcs after the local pairs, then every pair's least
         // distance (records sorted by (u, v) and distance; the first of each (u, v) kept)
-        uint64_t cap = std::max<uint64_t>(local + nh * 2, 1 << 16), m = 0;
+        uint64_t cap = std::max<uint64_t>({local + nh * 2, h->candidates + h->candidates / 8, 1 << 16}), m = 0;
         unsigned long long *mk0 = nullptr;
         uint32_t *md0 = nullptr;
         for (;;) {
@@ -6157,14 +6586,14 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
             RN_CUDA(cudaGetLastError());
             counts();
             m = h->count_host[0];
+            h->candidates = m;
             if (m <= cap) break;
             cap = m + m / 4;
         }
         unsigned long long *mk1 = h->get<unsigned long long>("m_key2", m);
         uint32_t *md1 = h->get<uint32_t>("m_d2", m);
         sh.clear();
-        add_shifts(&sh, 0, uint32_t(dbits), 64);  // distance
-        add_shifts(&sh, 0, 2 * vbits);           // (u, v)
+        add_shifts(&sh, 0, 2 * vbits);  // (u, v); each run's least distance is found as it is compacted
         const auto msrt = sort_kv(ws, mk0, md0, mk1, md1, m, sh, st);
         uint32_t *first = h->get<uint32_t>("first", m + 1), *first_at = h->get<uint32_t>("first_at", hist_words(m + 1));
         unsigned long long *uk = h->get<unsigned long long>("u_key", m);
@@ -6179,6 +6608,7 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
             uint32_t *tot = reinterpret_cast<uint32_t *>(h->count_host);
             RN_CUDA(cudaMemcpyAsync(&tot[0], first_at + m, 4, cudaMemcpyDeviceToHost, st));
             RN_CUDA(cudaStreamSynchronize(st));
+            late_check(ws);
             nu = tot[0];
             RN_CUDA(cudaGetLastError());
         }
@@ -6611,7 +7041,12 @@ static void batch_finish(Batch *b, uint64_t total, cudaStream_t st) {
     const uint32_t nblocks = uint32_t((total + RS_TILE - 1) / RS_TILE);
     unsigned long long *ki = b->keyA, *ko = b->keyB;
     uint32_t *vi = b->valA, *vo = b->valB;
-    for (uint32_t sh = 0; sh < 2 * b->vbits; sh += 8) {
+    std::vector<int> shifts;
+    for (uint32_t sh = 0; sh < 2 * b->vbits; sh += 8) shifts.push_back(int(sh));
+    const bool sweep = sweeps(total, shifts.size());
+    if (sweep)
+        sweep_sort(ki, vi, ko, vo, total, shifts, b->hist, b->out_u, b->out_v, b->out_d, b->vbits, 0xFFFFFFFFu, b->ws->ctl, st);
+    for (uint32_t sh = 0; sh < 2 * b->vbits && !sweep; sh += 8) {
         const bool last = sh + 8 >= 2 * b->vbits;
         k_rs_hist<<<nblocks, RS_THREADS, 0, st>>>(ki, vi, total, int(sh), b->hist, nblocks);
         scan_hist(b->hist, nblocks * 256, st);
@@ -6713,11 +7148,10 @@ static uint64_t batch_run_eager(Batch *b, cudaStream_t st) {
             b->out_d = (uint32_t *)device_alloc(b->out_cap * 4);
             batch_drop_graph(b);
         }
-        const uint32_t nblocks = uint32_t((b->total + RS_TILE - 1) / RS_TILE);
-        if (b->hist_cap < hist_words(uint64_t(nblocks) * 256)) {
+        if (b->hist_cap < sort_words(b->total)) {
             device_free(b->hist);
             b->hist = nullptr;
-            b->hist_cap = hist_words(uint64_t(nblocks) * 256);
+            b->hist_cap = sort_words(b->total);
             b->hist = (uint32_t *)device_alloc(b->hist_cap * 4);
             batch_drop_graph(b);
         }
@@ -6725,7 +7159,7 @@ static uint64_t batch_run_eager(Batch *b, cudaStream_t st) {
         std::vector<unsigned long long> po(b->off.begin(), b->off.end());
         RN_CUDA(cudaMemcpyAsync(b->pair_off_d, po.data(), po.size() * 8, cudaMemcpyHostToDevice, st));
         batch_finish(b, b->total, st);
-        RN_CUDA(cudaStreamSynchronize(st));  // po is a host temporary
+        check_control(read_control(b->ws, st));  // (po is a host temporary)
         b->stats.eager_runs++;
         return retried;
     }
@@ -6758,7 +7192,8 @@ void batch_run(Batch *b, void *user_stream, bool use_graph) {
         RN_CUDA(cudaGraphLaunch(b->exec, st));
         const Control c = read_control(b->ws, st);
         b->stats.graph_runs++;
-        if (!c.err && !c.n_failed && c.pairs == b->exec_pairs) {
+        check_control(c);
+        if (!c.n_failed && c.pairs == b->exec_pairs) {
             b->total = c.pairs;
             done = true;
         } else {
@@ -6770,7 +7205,8 @@ void batch_run(Batch *b, void *user_stream, bool use_graph) {
         const uint64_t retried = batch_run_eager(b, st);
         const uint32_t passes = (2 * b->vbits + 7) / 8;
         const uint64_t entries = (b->total + RS_TILE - 1) / RS_TILE * 256;
-        b->stats.launches_per_run = b->ws->launches + passes * (entries <= 2 * SCAN_CHUNK ? 3 : 5) + 1;
+        b->stats.launches_per_run =
+            b->ws->launches + (sweeps(b->total, passes) ? passes + 1 : passes * (entries <= 2 * SCAN_CHUNK ? 3 : 5)) + 1;
         if (retried || !b->laid_out_by_cost) {
             // the next run starts with fitting maps and the measured tile order
             batch_adapt_maps(b);

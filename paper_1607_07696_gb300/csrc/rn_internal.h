@@ -218,6 +218,7 @@ void set_allocator(rn_alloc_fn alloc, rn_free_fn free, void *ctx);
 void *device_alloc(size_t bytes);
 void device_free(void *p);
 void stream_sync(void *stream);
+void triple_to_host(const uint32_t *u, const uint32_t *v, const uint32_t *d, uint64_t n, uint32_t *dst, void *stream);
 
 }  // namespace rn
 

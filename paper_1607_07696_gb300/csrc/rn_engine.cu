@@ -656,6 +656,7 @@ struct SearchArgs {
     // overflow rows'), pages, table buckets, queue entries and words of a group's map,
     // groups resident on an SM
     const uint4 *__restrict__ ell;
+    uint32_t *next;  // its work counter (the control block's tile_next, or one of a batch's)
     uint32_t n_rows, pg_cap, pg_buckets, pg_queue, pg_words, pg_resident;
 };
 
@@ -1531,15 +1532,15 @@ __global__ void __launch_bounds__(32 * W * pg_groups(W), 32 / (W * pg_groups(W))
     for (;;) {
         uint32_t item = ahead;
         if (W == 1) {
-            if (ahead == PG_NONE && lane == 0) item = atomicAdd(&a.ctl->tile_next, 1u);
+            if (ahead == PG_NONE && lane == 0) item = atomicAdd(a.next, 1u);
             item = __shfl_sync(FULL, item, 0);
             ahead = PG_NONE;
             if (item < early) {
                 ahead = 0;  // (lane 0's alone is read)
-                if (lane == 0) ahead = atomicAdd(&a.ctl->tile_next, 1u);
+                if (lane == 0) ahead = atomicAdd(a.next, 1u);
             }
         } else {
-            if (gt == 0) ctl[PC_ITEM] = atomicAdd(&a.ctl->tile_next, 1u);
+            if (gt == 0) ctl[PC_ITEM] = atomicAdd(a.next, 1u);
             __syncthreads();
             item = ctl[PC_ITEM];
         }
@@ -4249,6 +4250,7 @@ static void page_launch(const DeviceGraph &g, uint32_t cap, SearchArgs a, uint32
     const PageShape p = page_shape(cap, items, ws->num_sms, hier);
     if (!g.ell) fail(RN_EINTERNAL, "search by pages without rows");
     a.ell = g.ell;
+    if (!a.next) a.next = &a.ctl->tile_next;
     a.n_rows = uint32_t(g.n + g.nvirt);
     a.pg_cap = p.cap;
     a.pg_buckets = p.buckets;
@@ -4437,7 +4439,9 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
             ws->ball_theta = std::max<uint32_t>(theta, 1);
             ws->ball_max = ball;
             ws->ball_mean = mean;
-            ws->page_max = std::max(pages, 0.97 * was);
+            // (at most 15% over this search's: scaled up with the square of the radius and down with
+            // less, a remembered count would grow with every change of the bound)
+            ws->page_max = std::min(std::max(pages, 0.97 * was), 1.15 * pages);
         }
     };
     if (!c.n_failed || c.err || c.check[0]) {
@@ -6750,7 +6754,12 @@ uint32_t plan_tile_src(const BatchPlan &p) { return std::max<uint32_t>(1, p.T / 
 // The smallest warp map whose 7/8 holds a ball of `ball` nodes with room to spare, or 0
 // when even the largest does not.
 uint32_t warp_map_for_ball(double ball, bool paged) {
-    if (paged) return page_class(ball) <= PG_MAX ? page_class(ball) : 0;  // (the ball's pages)
+    if (paged) {
+        // the ball's pages, in classes twice apart: fewer launches, each with more sources
+        for (uint32_t c = 16; c <= 1024; c *= 2)
+            if (ball <= c) return c;
+        return ball <= PG_MAX ? PG_MAX : 0;
+    }
     for (uint32_t ms = SRC_MS_MIN; ms <= SRC_MS_MAX; ms *= 2)
         if (ball <= src_fit(ms)) return ms;
     return 0;
@@ -6830,6 +6839,8 @@ uint32_t tune_cache_load(const char *path) {
     return uint32_t(plans.size());
 }
 
+constexpr uint32_t BATCH_SIDE = 4;
+
 struct Batch {
     int device = 0;
     uint32_t nq = 0, n_u = 0, pad = 0, vbits = 1;
@@ -6866,6 +6877,11 @@ struct Batch {
     uint64_t total = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    // the searches by pages of a recorded run go side by side: a work counter for each group,
+    // side streams and the events that fork and join them
+    uint32_t *next = nullptr;
+    cudaStream_t side[BATCH_SIDE] = {};
+    cudaEvent_t forked = nullptr, joined[BATCH_SIDE] = {};
     uint64_t exec_pairs = 0;
     rn_batch_stats stats{};
 };
@@ -6893,6 +6909,12 @@ void batch_destroy(Batch *b) {
                     (void *)b->valA, (void *)b->valB, (void *)b->hist, (void *)b->out_u, (void *)b->out_v,
                     (void *)b->out_d, (void *)b->ug.row_ptr, (void *)b->ug.adj, (void *)b->ug.iperm, (void *)b->ug.ell})
         device_free(p);
+    device_free(b->next);
+    for (cudaStream_t s : b->side)
+        if (s) cudaStreamDestroy(s);
+    for (cudaEvent_t e : b->joined)
+        if (e) cudaEventDestroy(e);
+    if (b->forked) cudaEventDestroy(b->forked);
     if (b->stream) cudaStreamDestroy(b->stream);
     workspace_destroy(b->ws);
     delete b;
@@ -7088,9 +7110,10 @@ static void batch_counts(Batch *b, cudaStream_t st) {
 }
 
 // The first launch of one group (the capturable part of its search).
-static void batch_launch_group(Batch *b, const Batch::Group &g, cudaStream_t st) {
+static void batch_launch_group(Batch *b, const Batch::Group &g, cudaStream_t st, uint32_t *next = nullptr) {
     if (!g.tiles) return;
     SearchArgs a = batch_args(b, g);
+    a.next = next;
     a.slab = b->ws->sh->slab;
     a.failed = b->ws->failed;
     a.ntiles = g.tiles;
@@ -7168,10 +7191,29 @@ static uint64_t batch_run_eager(Batch *b, cudaStream_t st) {
 // The capturable sequence: clears, one launch per group, sort and shift.
 static void batch_record(Batch *b, cudaStream_t st) {
     batch_clear(b, st);
+    // the searches by pages touch nothing that another group does (but counters that add up),
+    // so they fork onto the side streams, where one group's last sources overlap the next
+    // group's; tile groups share the slab and stay one after another
+    const size_t ng = b->groups.size();
+    const bool fork = b->paged && ng > 1;
+    if (fork) {
+        RN_CUDA(cudaMemsetAsync(b->next, 0, ng * 4, st));
+        RN_CUDA(cudaEventRecord(b->forked, st));
+        for (uint32_t i = 0; i < BATCH_SIDE; i++) RN_CUDA(cudaStreamWaitEvent(b->side[i], b->forked, 0));
+        uint32_t turn = 0;
+        for (size_t i = 0; i < ng; i++)
+            if (b->groups[i].T == 1) batch_launch_group(b, b->groups[i], b->side[turn++ % BATCH_SIDE], b->next + i);
+    }
     for (const auto &g : b->groups) {
-        RN_CUDA(cudaMemsetAsync(&b->ws->ctl->tile_next, 0, 8, st));
+        if (fork && g.T == 1) continue;
+        RN_CUDA(cudaMemsetAsync(&b->ws->ctl->tile_next, 0, 4, st));
         batch_launch_group(b, g, st);
     }
+    if (fork)
+        for (uint32_t i = 0; i < BATCH_SIDE; i++) {
+            RN_CUDA(cudaEventRecord(b->joined[i], b->side[i]));
+            RN_CUDA(cudaStreamWaitEvent(st, b->joined[i], 0));
+        }
     batch_finish(b, b->exec_pairs, st);
 }
 
@@ -7215,6 +7257,16 @@ void batch_run(Batch *b, void *user_stream, bool use_graph) {
         } else if (use_graph && !b->exec) {
             b->exec_pairs = b->total;
             ensure_slist(b->ws);  // allocates nothing inside the capture
+            device_free(b->next);
+            b->next = nullptr;
+            b->next = (uint32_t *)device_alloc(std::max<size_t>(b->groups.size(), 1) * 4);
+            if (!b->forked) {
+                RN_CUDA(cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming));
+                for (uint32_t i = 0; i < BATCH_SIDE; i++) {
+                    RN_CUDA(cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking));
+                    RN_CUDA(cudaEventCreateWithFlags(&b->joined[i], cudaEventDisableTiming));
+                }
+            }
             RN_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
             try {
                 batch_record(b, st);

@@ -101,3 +101,23 @@ def test_points_rejected(rn):
     # points on a path: distances are gaps between positions
     u, v, d = rn.rn_distance_join_points(g, [(0, 1, 1), (2, 3, 5)], [(1, 2, 3), (3, 2, 0)], rn.RN_INF)
     assert list(zip(u.tolist(), v.tolist(), d.tolist())) == [(0, 0, 6), (0, 1, 14), (1, 0, 8), (1, 1, 0)]
+
+
+@pytest.mark.parametrize("n", [2048, 2049])
+def test_points_staged_sizes(rn, oracle, n):
+    """One graph's staging over queries that grow, shrink and have an empty side, at node counts
+    on both sides of a sort digit, with most points of a query on a few edges."""
+    rng = np.random.default_rng(n)
+    e = I.road_graph(n, int(2.6 * n), n)
+    best = pins.least_weights(e)
+    few = list(best)[:3]
+    g = rn.rn_graph_load(e.src, e.dst, e.w, e.n)
+    og = oracle.graph(e.n, e.src, e.dst, e.w)
+    theta = 4 * int(np.median(e.w))
+    for nR, nS in ((0, 5), (5, 0), (1, 1), (300, 1), (3, 1500), (2, 2), (700, 700)):
+        pts = pins.random_points(rng, best, nR + nS)
+        for i in range(0, nR + nS, 2):
+            a, b = few[i % 3]
+            pts[i] = (b, a, i % (best[(a, b)] + 1)) if i % 4 else (a, b, i % (best[(a, b)] + 1))
+        R, S = pts[:nR], pts[nR:]
+        assert same(rn.rn_distance_join_points(g, R, S, theta), og.join_points(R, S, theta)), (nR, nS)

@@ -320,8 +320,8 @@ def batch_leg(rn, steps: int, warmup: int, stream, flush) -> dict:
         "tuned": {1: f"one plan for all (tile width {int(s1['plan_tile_width'])}, buckets of "
                      f"{int(s1['plan_delta_mult'])} median weights, {int(s1['plan_tile_sources'])} sources "
                      f"per tile)",
-                  2: "plan per size class", 3: "the default plans (warp search for small balls, tiles of 8 "
-                                               "sources for large)"}.get(int(s1["tuned"]), "no"),
+                  2: "plan per size class", 3: "the default plans (search by sources, tiles of 8 "
+                                               "sources for balls past it)"}.get(int(s1["tuned"]), "no"),
     }
     del b0, b1
     return res
@@ -407,14 +407,14 @@ def large_balls_leg(rn, steps: int, stream, flush, peak: float, peak_kind: str) 
             "blocks_per_sm": int(st["blocks_per_sm"]), "launches": int(st["launches"]),
             "retried_tiles": int(st["retried_tiles"]),
             "roofline": dict(roofline(st, n, statistics.mean(search), "road1070k_large_balls", peak, peak_kind),
-                             kernel="k_source_coop")}
+                             kernel="k_source_search")}
 
 
 def hier_leg(rn, steps: int) -> dict:
     """The hierarchical variant (searches local to the parts of the partition hierarchy,
     the searches from the far ends of the arcs that leave a part shared by every source,
     min-plus combination) on the 264k-node join, at several part sizes, beside the flat
-    warp search on the same graph: device time per join (CUDA events inside the query),
+    search on the same graph: device time per join (CUDA events inside the query),
     pairs/s and the phase counters; every result checked equal to the flat join's."""
     import numpy as np
 

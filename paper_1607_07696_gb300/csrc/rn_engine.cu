@@ -1363,10 +1363,10 @@ __global__ void __launch_bounds__(THREADS, (THREADS == NARROW ? CTAS_PER_SM : 1)
 // reached, nodes met); the host searches it again with more pages or with the tile search.
 //
 // What bounds it is instruction issue and the latency of a round (one L2 trip for the rows,
-// then lookup and atomic in shared memory), not bandwidth: 1.07M-node join, 26.4M ball nodes
-// and 147M relaxed arcs in 1.2 ms, 0.91G warp instructions (6.2 an arc), 65% issue active.
+// then lookup and atomic in shared memory), not bandwidth: 1.07M-node join, 25.0M ball nodes
+// and 139M relaxed arcs in 1.07 ms, 0.89G warp instructions (6.4 an arc), 68% issue active.
 // Hashing every node instead (1.15G instructions, two probes chains and two atomics an arc,
-// CSR offsets before the arcs) took 1.48 ms there, 1.27 ms against 0.74 on the 264k-node join
+// CSR offsets before the arcs) took 1.48 ms there, 1.27 ms against 0.70 on the 264k-node join
 // and 2.32 against 1.09 with balls of 3,500 nodes (eight warps a ball).
 constexpr uint32_t PG_BITS = 11;  // a group's pages are numbered in 11 bits
 constexpr uint32_t PG_SLOT = (1u << PG_BITS) - 1;
@@ -6783,11 +6783,13 @@ constexpr BatchPlan BIG_PLAN{32, 4, 4};
 // Sources per tile of a plan (one for the warp search).
 uint32_t plan_tile_src(const BatchPlan &p) { return std::max<uint32_t>(1, p.T / p.src_div); }
 
-// The smallest warp map whose 7/8 holds a ball of `ball` nodes with room to spare, or 0
-// when even the largest does not.
+// The smallest map for a ball: by pages, of `ball` pages; hashed, the smallest warp map whose
+// 7/8 holds `ball` nodes with room to spare.  0 when even the largest does not.
 uint32_t warp_map_for_ball(double ball, bool paged) {
     if (paged) {
-        // the ball's pages, in classes twice apart: fewer launches, each with more sources
+        // the ball's pages, in classes twice apart: fewer launches, each with more sources (the
+        // single query's classes, a fifth to a third apart, took 2.95 ms for 20 towns of 1k to
+        // 50k nodes, one group after another; these, side by side, 2.41)
         for (uint32_t c = 16; c <= 1024; c *= 2)
             if (ball <= c) return c;
         return ball <= PG_MAX ? PG_MAX : 0;
@@ -7451,9 +7453,9 @@ Batch *batch_create(const std::vector<const DeviceGraph *> &graphs, const std::v
             b->theta[i] = theta[i] == RN_INF ? RN_THETA_MAX : theta[i];
             if (b->theta[i] > RN_THETA_MAX) fail(RN_EINVAL, "theta must be <= 2^31 or RN_INF");
             b->cls[i] = size_class(b->n[i], b->nR[i], b->theta[i], median_w[i]);
-            // the default plan: the warp search while the ball estimated from the bound
-            // fits a 2048-slot warp map (a dozen warps per SM or more), else tiles, whose
-            // sources share their searches' passes
+            // the default plan: the source search while the ball estimated from the bound is
+            // one a group's pages hold, or fits a 2048-slot warp map (a dozen warps per SM or
+            // more), else tiles, whose sources share their searches' passes
             if (graphs[i]->n < SK_NODE &&
                 first_ball_estimate(*graphs[i], b->theta[i], median_w[i]) <= (b->paged ? PG_BALL_MAX : src_fit(2048)))
                 b->plan[i] = WARP_PLAN;

@@ -7294,12 +7294,10 @@ void batch_run(Batch *b, void *user_stream, bool use_graph) {
             device_free(b->next);
             b->next = nullptr;
             b->next = (uint32_t *)device_alloc(std::max<size_t>(b->groups.size(), 1) * 4);
-            if (!b->forked) {
-                RN_CUDA(cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming));
-                for (uint32_t i = 0; i < BATCH_SIDE; i++) {
-                    RN_CUDA(cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking));
-                    RN_CUDA(cudaEventCreateWithFlags(&b->joined[i], cudaEventDisableTiming));
-                }
+            if (!b->forked) RN_CUDA(cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming));
+            for (uint32_t i = 0; i < BATCH_SIDE; i++) {
+                if (!b->side[i]) RN_CUDA(cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking));
+                if (!b->joined[i]) RN_CUDA(cudaEventCreateWithFlags(&b->joined[i], cudaEventDisableTiming));
             }
             RN_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
             try {

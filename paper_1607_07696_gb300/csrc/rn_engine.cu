@@ -3420,7 +3420,9 @@ static int attr_device() {
 // (each digit looks back on its own thread until a block whose running sum is known), orders
 // its records in shared memory and writes runs of equal digits.  Blocks take their number in
 // the order they start, so the ones looked back at run or have ended; a wait is cut after
-// about a second and reported as a failed check.
+// about a second and reported as a failed check.  A pass that finds a failed check writes
+// nothing: its input has gaps that hold other records, whose digits the counts (taken from the
+// sort's input) do not cover, so their places could lie past the buffers.
 constexpr uint64_t SWEEP_MIN = 1u << 18, SWEEP_FEW = 1u << 15;  // (SWEEP_FEW: from five passes on)
 constexpr uint64_t SWEEP_MAX = 1u << 30;  // counts leave two bits of their word for the kind
 constexpr int SWEEP_THREADS = 512, SWEEP_WARPS = SWEEP_THREADS / 32;
@@ -3468,11 +3470,12 @@ __global__ void __launch_bounds__(SWEEP_THREADS, 2) k_sweep(const unsigned long 
     __shared__ uint32_t s_block, s_scan[8], s_scan2[8], s_base[256], s_lost;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lt = (1u << lane) - 1;
     if (tid == 0) {
+        s_lost = __ldcg(&ctl->check[0]);  // (a pass gave up: this one's input has gaps)
         s_block = atomicAdd(ticket, 1u);
-        s_lost = 0;
     }
     for (uint32_t i = tid; i < SWEEP_WARPS * 256; i += SWEEP_THREADS) wcnt[0][i] = 0;
     __syncthreads();
+    if (s_lost) return;
     const uint32_t block = s_block;
     const uint64_t first = uint64_t(block) * SWEEP_TILE + uint64_t(warp) * (SWEEP_ROUNDS * 32);
     unsigned long long k[SWEEP_ROUNDS];
@@ -3565,7 +3568,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS, 2) k_sweep(const unsigned long 
         s_base[tid] = global + before - local;  // (a record's place is this plus its place in the block)
     }
     __syncthreads();
-    if (s_lost) return;  // (nothing is written past the records)
+    if (s_lost) return;  // (its tile stays unwritten: the passes behind this one see the check and stop)
 #pragma unroll
     for (int r = 0; r < SWEEP_ROUNDS; r++) {
         if (first + uint64_t(r) * 32 + lane < n) {
@@ -7569,3 +7572,46 @@ void batch_pairs_dev(const Batch *b, uint32_t i, const uint32_t **u, const uint3
 const rn_batch_stats &batch_stats(const Batch *b) { return b->stats; }
 
 }  // namespace rn
+
+#ifdef RN_CHECKS
+// For the checked build's tests: the words that a sort of n records changes in its other buffers
+// and its result when the control block holds a failed check, as it does for the passes behind
+// one that gave up a wait.
+extern "C" int rn_checks_sort_after_failure(uint64_t n, uint64_t *changed) {
+    using namespace rn;
+    constexpr uint32_t VBITS = 20;
+    constexpr uint64_t ROOM = 1024;  // words past the records
+    void *key = nullptr, *val = nullptr, *rest = nullptr, *hist = nullptr, *ctl = nullptr;
+    int status = RN_OK;
+    try {
+        if (!sweeps(n, 5)) fail(RN_EINVAL, "not a size that is sorted in single-launch passes");
+        std::vector<uint64_t> k(n);
+        std::vector<uint32_t> out(6 * n + ROOM, 0xA5A5A5A5u);
+        for (uint64_t i = 0; i < n; i++) k[i] = (i * 0x9E3779B97F4A7C15ull) >> (64 - 2 * VBITS);
+        Control c{};
+        c.check[0] = 32;
+        key = device_alloc(n * 8);
+        val = device_alloc(n * 4);
+        rest = device_alloc(out.size() * 4);  // the other keys and values, then u, v and d
+        hist = device_alloc(sort_words(n) * 4);
+        ctl = device_alloc(sizeof(Control));
+        RN_CUDA(cudaMemcpy(key, k.data(), n * 8, cudaMemcpyHostToDevice));
+        RN_CUDA(cudaMemset(val, 0, n * 4));
+        RN_CUDA(cudaMemcpy(rest, out.data(), out.size() * 4, cudaMemcpyHostToDevice));
+        RN_CUDA(cudaMemcpy(ctl, &c, sizeof(c), cudaMemcpyHostToDevice));
+        RN_CUDA(cudaDeviceSynchronize());
+        uint32_t *r = static_cast<uint32_t *>(rest);
+        sweep_sort(static_cast<unsigned long long *>(key), static_cast<uint32_t *>(val),
+                   reinterpret_cast<unsigned long long *>(r), r + 2 * n, n, {0, 8, 16, 24, 32}, static_cast<uint32_t *>(hist),
+                   r + 3 * n, r + 4 * n, r + 5 * n, VBITS, 0xFFFFFFFFu, static_cast<Control *>(ctl), nullptr);
+        RN_CUDA(cudaDeviceSynchronize());
+        RN_CUDA(cudaMemcpy(out.data(), rest, out.size() * 4, cudaMemcpyDeviceToHost));
+        *changed = 0;
+        for (uint32_t x : out) *changed += x != 0xA5A5A5A5u;
+    } catch (const Error &e) {
+        status = e.status;
+    }
+    for (void *p : {key, val, rest, hist, ctl}) device_free(p);
+    return status;
+}
+#endif

@@ -4201,6 +4201,9 @@ static uint32_t page_class(double pages) {
     return PG_MAX + 1;
 }
 
+// The hierarchical variant's local searches: one warp a source up to this many pages, else four.
+constexpr uint32_t HIER_WARP_PAGES = 96, HIER_WARPS = 4;
+
 struct PageShape {
     uint32_t cap, buckets, queue, words, warps, blocks, groups;  // blocks, groups: per SM
     size_t smem;
@@ -4230,7 +4233,7 @@ static PageShape page_shape(uint32_t cap, uint32_t items, int sms, bool hier) {
         p.smem = size_t(p.words) * 4 * G;
         p.blocks = std::min<uint32_t>(uint32_t(233472 / (p.smem + 1024 + 256)), 32 / (W * G));
         p.groups = p.blocks * G;
-        if (hier ? (W == 4 || (W == 1 && cap <= 96)) : p.blocks && (W >= most || W * std::min(p.groups, want) >= (W == 1 ? 16u : 28u))) break;
+        if (hier ? (W == HIER_WARPS || (W == 1 && cap <= HIER_WARP_PAGES)) : p.blocks && (W >= most || W * std::min(p.groups, want) >= (W == 1 ? 16u : 28u))) break;
     }
     if (!p.blocks) fail(RN_EINTERNAL, "a group's pages do not fit an SM");
     return p;
@@ -4264,7 +4267,7 @@ static void page_launch(const DeviceGraph &g, uint32_t cap, SearchArgs a, uint32
     const uint32_t grid = std::max<uint32_t>(1, std::min<uint32_t>((items + G - 1) / G, uint32_t(ws->num_sms) * p.blocks));
     if (hier) {
         if (p.warps == 1) launch_pages<1, true>(a, p, grid, st);
-        else launch_pages<4, true>(a, p, grid, st);
+        else launch_pages<HIER_WARPS, true>(a, p, grid, st);
     } else {
         switch (p.warps) {
             case 1: launch_pages<1, false>(a, p, grid, st); break;
@@ -6349,9 +6352,12 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
     for (uint32_t m = SRC_MS_MIN; m <= SRC_MS_MAX && !map_slots; m *= 2)
         if (double(max_part) <= src_fit(m)) map_slots = m;
     if (!map_slots) fail(RN_EINVAL, "the hierarchical variant takes parts of at most 6516 nodes");
-    // by pages: the part's consecutive ids, and its overflow rows' (consecutive too)
+    // by pages: the part's consecutive ids, and its overflow rows' (consecutive too), each of
+    // which may begin and end inside a page; where warps share the map, also a page for every
+    // warp, which may hold a slot that it drew for a page another warp inserted first
     const uint32_t part_virt = uint32_t(std::min<uint64_t>(g.nvirt, uint64_t(max_part) * g.row_chain));
-    const uint32_t part_pages = std::max<uint32_t>(8, (max_part + 31) / 32 + (part_virt + 31) / 32 + 2);
+    uint32_t part_pages = std::max<uint32_t>(8, (max_part + 31) / 32 + (part_virt + 31) / 32 + 2);
+    if (part_pages > HIER_WARP_PAGES) part_pages += HIER_WARPS;
     std::lock_guard<std::mutex> device_lock(ws->sh->mu);
     Range range("rn.hier");
     *stats = rn_query_stats{};

@@ -6476,7 +6476,10 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
             a.brd_d = brd_d;
             a.brd_cap = brd_cap;
             a.brd_count = h->count;
-            if (nR) source_launch(g, by_pages(g, bnd), by_pages(g, bnd) ? part_pages : map_slots, a, nR, ws, st, true);
+            // (hashed where a part's pages, counted with the most overflow rows its nodes could
+            // have, are more than a group's map holds)
+            const bool paged = by_pages(g, bnd) && part_pages <= PG_MAX;
+            if (nR) source_launch(g, paged, paged ? part_pages : map_slots, a, nR, ws, st, true);
             c = read_control(ws, st);
             counts();
             check_control(c);

@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -3608,6 +3609,11 @@ static bool sweeps(uint64_t n, size_t passes) {
 // The sort of (k0, v0) by the listed digits in single-launch passes, with (k1, v1) as the other
 // buffers; the last pass writes the struct-of-arrays result when out_u is given.  Returns the
 // kernels launched.
+#ifdef RN_CHECKS
+static std::atomic<int> g_fail_sort{0};  // the checked build's tests: the sort that finds a failed check
+__global__ void k_fail_check(Control *ctl) { record_check(ctl, 32, 0, 0); }
+#endif
+
 static uint32_t sweep_sort(unsigned long long *k0, uint32_t *v0, unsigned long long *k1, uint32_t *v1, uint64_t n,
                            const std::vector<int> &shifts, uint32_t *hist, uint32_t *out_u, uint32_t *out_v, uint32_t *out_d,
                            uint32_t vbits, uint32_t umask, Control *ctl, cudaStream_t st) {
@@ -3620,6 +3626,9 @@ static uint32_t sweep_sort(unsigned long long *k0, uint32_t *v0, unsigned long l
     SweepShifts sh{};
     sh.n = int(passes);
     for (uint32_t p = 0; p < passes; p++) sh.shift[p] = shifts[p];
+#ifdef RN_CHECKS
+    if (g_fail_sort > 0 && --g_fail_sort == 0) k_fail_check<<<1, 1, 0, st>>>(ctl);
+#endif
     RN_CUDA(cudaMemsetAsync(hist, 0, (SWEEP_HEAD + size_t(nb) * 256 * passes) * 4, st));
     k_sweep_count<<<std::min<uint32_t>(nb, 1024), 256, 0, st>>>(k0, v0, n, sh, hist);
     for (uint32_t p = 0; p < passes; p++) {
@@ -6606,6 +6615,7 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
             ws->launches++;
         }
         lap(1);
+        late_check(ws);  // (the sort of the hits, before they are used)
         mark();
         // 4. candidates through the exit arcs after the local pairs, then every pair's least
         // distance (records sorted by (u, v) and distance; the first of each (u, v) kept)
@@ -6709,6 +6719,7 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
     out->n = np;
     RN_CUDA(cudaEventRecord(ws->ev1, st));
     RN_CUDA(cudaEventSynchronize(ws->ev1));
+    late_check(ws);
     float ms = 0;
     RN_CUDA(cudaEventElapsedTime(&ms, ws->ev0, ws->ev1));
     stats->pairs = np;
@@ -7623,4 +7634,8 @@ extern "C" int rn_checks_sort_after_failure(uint64_t n, uint64_t *changed) {
     for (void *p : {key, val, rest, hist, ctl}) device_free(p);
     return status;
 }
+
+// For the checked build's tests: the nth sort by single-launch passes from now on finds a failed check,
+// as behind a wait that was cut.  Returns how many of the last setting were left.
+extern "C" int rn_checks_fail_sort(int nth) { return rn::g_fail_sort.exchange(nth); }
 #endif

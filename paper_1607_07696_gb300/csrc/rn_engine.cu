@@ -354,8 +354,8 @@ struct Workspace {
     unsigned long long *mq_counts = nullptr;
     uint8_t *mq_swap = nullptr;  // per query: searched from S
     uint64_t mq_cap_q = 0, mq_cap_bits = 0, mq_cap_sids = 0;
-    // the largest source ball the last warp search met (or estimated, for sources
-    // whose map overflowed) and its bound: predicts the next query's balls
+    // the largest source ball the last source search met (or estimated, for sources that went
+    // to the tile search), the mean ball, and its bound: predicts the next query's balls
     double ball_max = 0, ball_mean = 0, page_max = 0;
     uint32_t ball_theta = 0;
     // warp search: per source its first pair and pair count; whether the last search
@@ -4443,9 +4443,12 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
     ws->src_clean = !c.n_failed && !c.err && !c.check[0];
     ws->blocks_per_sm = !nsrc ? 0 : paged ? int(page_shape(ms0, nsrc, ws->num_sms, false).blocks) : source_blocks_per_sm(ms0);
     double ball = c.src_max_ball, pages = c.src_max_pages;
-    // mean ball of the sources the first pass completed (0 when none did)
-    const double mean = nsrc > c.n_failed ? double(c.slots) / double(nsrc - c.n_failed) : 0.0;
+    // nodes met by all sources: of those that a map held as counted, of those that went to tiles as
+    // estimated (the mean of the sources that the first pass completed alone would be that of its
+    // smallest balls, down to a handful of nodes, and k closest pairs sizes its first radius by it)
+    double met = double(c.slots);
     auto learn = [&] {
+        const double mean = nsrc ? met / double(nsrc) : 0.0;
         // (k closest pairs lowers its bound as it goes: its balls say nothing of theta)
         if (learn_balls && nsrc && ball >= 64) {  // a handful of nodes says little about the growth
             // (the most pages of the last searches, scaled to this bound: other sets' largest
@@ -4470,10 +4473,14 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
     };
     std::map<uint32_t, std::vector<uint4>> grow;  // warp map -> its sources (index, 0, 0, 0)
     std::vector<uint4> to_tiles;
-    double tile_est = 0;
+    double tile_est = 0, tile_met = 0;
+    auto tiles = [&](const uint4 &f, double e) {
+        to_tiles.push_back(f);
+        tile_est = std::max(tile_est, e);
+        tile_met += e;
+    };
     auto route = [&](const uint4 &f, uint32_t failed_at) {
         const double e = estimate(f);
-        ball = std::max(ball, e);
         if (paged) {
             // its pages, in proportion to the nodes met when they were used up
             const double need = double(failed_at) * std::max(1.3, 1.15 * e / double(std::max<uint32_t>(f.w, 1)));
@@ -4482,8 +4489,7 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
                 pages = std::max<double>(pages, std::min(need, double(PG_MAX)));
                 grow[size].push_back(make_uint4(f.x, 0, 0, 0));
             } else {
-                to_tiles.push_back(f);
-                tile_est = std::max(tile_est, e);
+                tiles(f, e);
             }
             return;
         }
@@ -4492,8 +4498,7 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
         if (ms <= SRC_MS_MAX) {
             grow[ms].push_back(make_uint4(f.x, 0, 0, 0));
         } else {
-            to_tiles.push_back(f);
-            tile_est = std::max(tile_est, e);
+            tiles(f, e);
         }
     };
     for (const uint4 &f : read_ranges(ws->failed, c.n_failed, st)) route(f, ms0);
@@ -4516,6 +4521,8 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
         pages = std::max<double>(pages, c.src_max_pages);
         for (const uint4 &f : read_ranges(ws->failed, c.n_failed, st)) route(f, ms);
     }
+    ball = std::max(ball, tile_est);
+    met = double(c.slots) + tile_met;
     ws->src_tiles = !to_tiles.empty();
     if (!to_tiles.empty()) {
         // consecutive sources of one query become ranges of up to T sources each

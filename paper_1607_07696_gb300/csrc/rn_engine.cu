@@ -4422,7 +4422,7 @@ static uint32_t source_first_map(const DeviceGraph &g, const Workspace *ws, uint
 static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs a, uint32_t nsrc, uint32_t ms0,
                                  uint32_t T, uint32_t theta, const std::vector<uint32_t> &inst_first,
                                  cudaStream_t st, uint64_t *retried, bool learn_balls = true,
-                                 const std::function<void()> &after = {}) {
+                                 const std::function<void()> &after = {}, bool one_bound = true) {
     a.n_nodes = g.n;
     a.n_arcs = g.arcs;
     a.range_list = nullptr;
@@ -4448,7 +4448,9 @@ static Control source_search_all(const DeviceGraph &g, Workspace *ws, SearchArgs
     // smallest balls, down to a handful of nodes, and k closest pairs sizes its first radius by it)
     double met = double(c.slots);
     auto learn = [&] {
-        const double mean = nsrc ? met / double(nsrc) : 0.0;
+        // (several queries, each with its own bound: their mean is no ball's at the largest bound)
+        const double r = ws->ball_theta ? double(theta) / double(ws->ball_theta) : 0.0;
+        const double mean = !one_bound ? ws->ball_mean * r * r : nsrc ? met / double(nsrc) : 0.0;
         // (k closest pairs lowers its bound as it goes: its balls say nothing of theta)
         if (learn_balls && nsrc && ball >= 64) {  // a handful of nodes says little about the growth
             // (the most pages of the last searches, scaled to this bound: other sets' largest
@@ -4960,6 +4962,7 @@ void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg
     *stats = rn_query_stats{};
     uint32_t max_bound = 0;
     for (uint32_t t : theta) max_bound = std::max(max_bound, std::min(t, RN_THETA_MAX));
+    const bool one_bound = std::all_of(theta.begin(), theta.end(), [&](uint32_t t) { return t == theta[0]; });
     const bool by_source = use_source_search(g, ws, cfg, max_bound, median_w);
     const uint32_t delta = choose_delta(cfg, median_w, by_source);
     stats->tile_width = by_source ? 1 : T;
@@ -5097,7 +5100,8 @@ void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg
         early = true;
     };
     auto search_pass = [&] {
-        return by_source ? source_search_all(g, ws, a, total, ms0, T, max_bound, first, st, &retried, true, place_early)
+        return by_source ? source_search_all(g, ws, a, total, ms0, T, max_bound, first, st, &retried, true, place_early,
+                                             one_bound)
                          : search_all(g, ws, T, a, 0, st, &retried, cfg.map_slots, true, &ranges);
     };
     Control c = search_pass();

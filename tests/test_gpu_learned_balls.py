@@ -58,3 +58,23 @@ def test_after_a_first_search_that_few_sources_complete(rn, world, reorder, ball
     st = rn.rn_last_query_stats()
     assert st["tile_width"] == 1 and st["passes"] <= 2
     assert st["slots"] < 300 * 3 * ball
+
+
+@pytest.mark.parametrize("reorder,ball", [(True, 6000), (False, 4000)])
+def test_after_joins_of_several_bounds(rn, world, reorder, ball):
+    """Joins searched together, most of them with a small bound: their mean ball is not the one at
+    the largest bound."""
+    e, og = world
+    rng = np.random.default_rng(203)
+    R, S = sets(e, rng, 300, 400, 0)
+    theta = int(np.sort(og.sssp(int(R[-1]))[0])[ball])
+    small = int(np.sort(og.sssp(int(R[-1]))[0])[3])
+    P, Q = sets(e, rng, 4000, 4000, 0)
+    g = rn.rn_graph_load(e.src, e.dst, e.w, e.n, flags=rn.RN_UNDIRECTED | (rn.RN_REORDER if reorder else 0))
+    for run in range(2):
+        outs = rn.rn_join_many(g, [(P, Q, small), (R, S, theta)])
+        assert same(outs[0], og.join(P, Q, small)) and same(outs[1], og.join(R, S, theta)), run
+    assert same(rn.rn_kcp(g, R, S, 2_000), og.kcp(R, S, 2_000))
+    st = rn.rn_last_query_stats()
+    assert st["tile_width"] == 1 and st["passes"] <= 2
+    assert st["slots"] < 300 * 3 * ball

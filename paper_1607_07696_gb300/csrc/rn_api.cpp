@@ -99,7 +99,12 @@ void to_host_pairs(const rn_dpairs &d, rn_pairs *out, void *stream) {
     }
     if (d.n) {
         if (blk && d.n <= TO_HOST_MAX) {
-            triple_to_host(d.u, d.v, d.d, d.n, blk, stream);
+            try {
+                triple_to_host(d.u, d.v, d.d, d.n, blk, stream);
+            } catch (...) {
+                rn_pairs_free(out);  // (the block goes back to the pool)
+                throw;
+            }
         } else {
             cudaMemcpyAsync(out->u, d.u, d.n * 4, cudaMemcpyDeviceToHost, st);
             cudaMemcpyAsync(out->v, d.v, d.n * 4, cudaMemcpyDeviceToHost, st);

@@ -27,6 +27,7 @@ namespace rn {
 // keeps at most POOL_MAX bytes.
 namespace {
 constexpr size_t POOL_MAX = size_t(1) << 30;
+constexpr size_t POOL_BLOCK = size_t(1) << 16;  // the smallest block, for every result that it holds
 std::mutex g_pool_mu;
 std::multimap<size_t, void *> g_pool_free;        // capacity -> free block
 std::unordered_map<void *, size_t> g_pool_blocks;  // every block handed out or pooled
@@ -36,14 +37,14 @@ void *pinned_take(size_t bytes) {
     {
         std::lock_guard<std::mutex> lk(g_pool_mu);
         auto it = g_pool_free.lower_bound(bytes);
-        if (it != g_pool_free.end() && it->first <= 2 * bytes) {
+        if (it != g_pool_free.end() && it->first <= std::max(2 * bytes, POOL_BLOCK)) {
             void *p = it->second;
             g_pool_free_bytes -= it->first;
             g_pool_free.erase(it);
             return p;
         }
     }
-    size_t cap = 1 << 16;
+    size_t cap = POOL_BLOCK;
     while (cap < bytes) cap <<= 1;
     void *p = nullptr;
     if (cudaHostAlloc(&p, cap, cudaHostAllocPortable) != cudaSuccess || !p) {

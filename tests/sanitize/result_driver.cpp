@@ -1,5 +1,5 @@
-// A result whose copy to the host fails goes back to the pool of page-locked blocks: rn_api.cpp over
-// fakes of the calls that a result makes, the copying launch failing.  Built as a shared library
+// Results and the pool of page-locked blocks: rn_api.cpp over fakes of the calls that a result makes,
+// the copying launch failing or not.  Built as a shared library
 // (the engine's functions stay unresolved) and run by tests/test_host_result.py.
 #include <cstdlib>
 
@@ -8,6 +8,7 @@
 #include "rn_internal.h"
 
 static int allocations = 0;
+static bool fails = true;  // the copying launch
 
 extern "C" cudaError_t cudaHostAlloc(void **p, size_t bytes, unsigned) {
     allocations++;
@@ -25,7 +26,7 @@ extern "C" cudaError_t cudaMemcpyAsync(void *, const void *, size_t, cudaMemcpyK
 namespace rn {
 void fail(rn_status s, const std::string &msg) { throw Error{s, msg}; }
 void triple_to_host(const uint32_t *, const uint32_t *, const uint32_t *, uint64_t, uint32_t *, void *) {
-    fail(RN_ECUDA, "launch failed");
+    if (fails) fail(RN_ECUDA, "launch failed");
 }
 void to_host_pairs(const rn_dpairs &d, rn_pairs *out, void *stream);
 }  // namespace rn
@@ -47,4 +48,18 @@ extern "C" int failed_results(int *blocks) {
     }
     *blocks = allocations;
     return bad;
+}
+
+// The blocks allocated for `runs` results of n pairs, each freed before the next.
+extern "C" int blocks_for_results(uint64_t n, int runs) {
+    fails = false;
+    allocations = 0;
+    for (int run = 0; run < runs; run++) {
+        uint32_t word = 0;
+        rn_dpairs d{&word, &word, &word, n, n};
+        rn_pairs out{};
+        rn::to_host_pairs(d, &out, nullptr);
+        rn_pairs_free(&out);
+    }
+    return allocations;
 }

@@ -4143,7 +4143,12 @@ static void rows_copy(const DeviceGraph &g, uint32_t node_off, uint32_t virt_at,
 // Whether the graph is searched by pages, and its rows.  The pages pay where a ball fills
 // them: two arcs of five or more stay inside a page (a road network in bisection order: four
 // of five; random ids: none).  A hub would put its arcs into a long chain of overflow rows,
-// one round each, so graphs with nodes of more than 64 arcs keep the hashed search.
+// one round each, so graphs with nodes of more than 64 arcs keep the hashed search.  So do
+// graphs of more than three overflow rows to four nodes: every row is a node of its own in a
+// ball, and a round of its own behind the node's.  Seven joins each (2 to 20 hops, 500 to 20,000
+// sources) on planar graphs of 200,000 nodes took, by pages and hashed: with 0.64 rows a node
+// (9.2 arcs) 0.17 to 0.39 ms against 0.22 to 0.43, none slower; with 1.0 (10.3 arcs) 0.20 to 0.57
+// against 0.24 to 0.56, one slower by 15%; with 2.0 (17.8 arcs) 0.26 to 2.7 against 0.37 to 1.2, six slower.
 static void build_rows(const HostGraph &g, DeviceGraph *d) {
     uint64_t inside = 0, nvirt = 0;
     uint32_t max_deg = 0, max_w = 0;
@@ -4162,7 +4167,7 @@ static void build_rows(const HostGraph &g, DeviceGraph *d) {
         }
     }
     d->far = g.n ? uint64_t(g.n - 1) * max_w : 0;
-    d->paged = max_deg <= 64 && 5 * inside >= 2 * g.arcs() && g.n + nvirt <= PG_ROWS_MAX;
+    d->paged = max_deg <= 64 && 5 * inside >= 2 * g.arcs() && 4 * nvirt <= 3 * uint64_t(g.n) && g.n + nvirt <= PG_ROWS_MAX;
     if (!d->paged) return;
     d->nvirt = uint32_t(nvirt);
     d->row_chain = max_deg <= PG_ROW ? 0 : (max_deg - PG_ROW + PG_ROW - 2) / (PG_ROW - 1);

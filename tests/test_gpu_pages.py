@@ -104,3 +104,26 @@ def test_longest_distances(rn, oracle, theta):
         ref = og.join(R, S, min(theta, rn.RN_THETA_MAX))
         assert same(rn.rn_distance_join(g, R, S, theta), ref), T
         assert same(rn.rn_kcp(g, R, S, 500, theta), og.kcp(R, S, 500, min(theta, rn.RN_THETA_MAX))), T
+
+
+@pytest.mark.parametrize("k,paged", [(5, True), (8, True), (10, False), (16, False)])
+def test_dense_graphs(rn, oracle, k, paged):
+    """Planar graphs around the most overflow rows a node that the search by pages takes (three to
+    four nodes): rows are held, 64 bytes a node and overflow row, where it does."""
+    rng = np.random.default_rng(k)
+    xy = rng.random((12_000, 2))
+    ab = I._knn_edges(I._knn_table(xy, k), k)
+    w = rng.integers(1, 300, size=len(ab))
+    deg = np.bincount(ab.ravel(), minlength=len(xy))
+    rows = int(((np.maximum(deg, 8) - 8 + 6) // 7).sum())
+    assert (4 * rows <= 3 * len(xy)) == paged
+    og = oracle.graph(len(xy), ab[:, 0], ab[:, 1], w)
+    g, plain = (rn.rn_graph_load(ab[:, 0], ab[:, 1], w, len(xy), flags=rn.RN_UNDIRECTED | f) for f in (rn.RN_REORDER, 0))
+    held = rn.rn_graph_info(g)["device_bytes"] - rn.rn_graph_info(plain)["device_bytes"]
+    assert held == (64 * (len(xy) + rows) if paged else 0)
+    R, S = I.disjoint_sets(len(xy), 700, 900, k)
+    for theta in (150, 700):
+        ref = og.join(R, S, theta)
+        for run in range(2):
+            assert same(rn.rn_distance_join(g, R, S, theta), ref), (theta, run)
+    assert same(rn.rn_kcp(g, R, S, 3_000), og.kcp(R, S, 3_000))

@@ -4587,6 +4587,18 @@ static bool can_place(const Workspace *ws, const Control &c) {
     return !ws->src_tiles && c.max_seg <= PLACE_MAX && c.pairs <= ws->pair_cap && c.pairs < 0xFFFFFFFFull;
 }
 
+static void ensure_place_state(Workspace *ws, uint32_t blocks, cudaStream_t st) {
+    if (ws->place_cap >= blocks) return;
+    device_free(ws->place_state);
+    ws->place_state = nullptr;
+    ws->place_cap = 0;
+    const uint32_t cap = std::max<uint32_t>(blocks, 1024);
+    ws->place_state = (unsigned long long *)device_alloc(size_t(cap) * 8);
+    ws->place_cap = cap;
+    RN_CUDA(cudaMemsetAsync(ws->place_state, 0, size_t(cap) * 8, st));
+    ws->place_epoch = 0;
+}
+
 // The canonical order by placement (k_place: source order is the output order): into `out`
 // or, with none, into the workspace's other (key, distance) records, in (u, v) order.  Before
 // the search's outcome is known (`early`) the kernel looks at it itself.
@@ -4594,14 +4606,7 @@ static void place_launch(Workspace *ws, uint32_t nsrc, uint32_t vbits, uint32_t 
                          cudaStream_t st, bool early) {
     if (!nsrc) return;
     const uint32_t nb = (nsrc + PLACE_SEGS - 1) / PLACE_SEGS;
-    if (ws->place_cap < nb) {
-        device_free(ws->place_state);
-        ws->place_state = nullptr;
-        ws->place_cap = std::max<uint32_t>(nb, 1024);
-        ws->place_state = (unsigned long long *)device_alloc(size_t(ws->place_cap) * 8);
-        RN_CUDA(cudaMemsetAsync(ws->place_state, 0, size_t(ws->place_cap) * 8, st));
-        ws->place_epoch = 0;
-    }
+    ensure_place_state(ws, nb, st);
     if (!early) RN_CUDA(cudaMemsetAsync(&ws->ctl->place_next, 0, 4, st));
     ws->place_epoch = (ws->place_epoch + 1) & 0x3FFFFFFFu;
     if (!ws->place_epoch) {  // (the epochs start again: no word of theirs may be left)
@@ -4679,25 +4684,6 @@ static void ensure_slab(Workspace *ws) {
     sh->slab_ctas = grid_max;
 }
 
-// Grow the workspace's buffers now for queries of up to max_r sources and max_pairs
-// pairs (raw pairs and their sort), so such queries allocate and free nothing later:
-// freeing device memory synchronises the whole device, which would stall every other
-// stream's work.
-void workspace_reserve(Workspace *ws, uint32_t max_r, uint64_t max_pairs) {
-    ensure_u32(&ws->rsorted, &ws->rsorted_cap, std::max<uint32_t>(max_r, 1));
-    ensure_ranges(&ws->failed, &ws->failed_cap, std::max<uint32_t>(max_r, 1));
-    ensure_ranges(&ws->failed2, &ws->failed2_cap, std::max<uint32_t>(max_r, 1));
-    ensure_pairs(ws, max_pairs);
-    grow(ws, &ws->hist, &ws->hist_cap, sort_words(max_pairs), 4);
-    ensure_slist(ws);
-    if (!ws->seg || ws->seg_cap < max_r) {  // the warp search's per-source segments
-        device_free(ws->seg);
-        ws->seg = nullptr;
-        ws->seg_cap = std::max<uint32_t>(max_r, 1024);
-        ws->seg = (uint2 *)device_alloc(size_t(ws->seg_cap) * 8);
-    }
-}
-
 static uint32_t mark_sets(const uint32_t *dR, uint32_t nR, const uint32_t *dS, uint32_t nS, const DeviceGraph &g,
                           uint32_t *used, uint32_t *rbits, uint32_t *sbits, Control *ctl, bool by_orig, cudaStream_t st) {
     const uint64_t ids = uint64_t(nR) + nS;
@@ -4750,6 +4736,13 @@ static bool search_from_s(const DeviceGraph &g, const EngineConfig &cfg, uint64_
         return true;
     }
     return g.symmetric && nS * 5 < nR * 4;
+}
+
+// Searches from S: room for the ranks of the marked ids.
+static void ensure_ranks(Workspace *ws) {
+    if (ws->ranks) return;
+    ws->ranks = (uint32_t *)device_alloc(std::max<size_t>(ws->nwords, 1) * 4);
+    ws->bytes += size_t(ws->nwords) * 4;
 }
 
 void run_join(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint32_t median_w,
@@ -4826,10 +4819,7 @@ void run_join(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint
     const uint32_t nranks = nR + nS;  // (ranks among all marked ids; S's have no pairs)
     const std::function<void()> place_early = [&] {
         if (by_rank) {
-            if (!ws->ranks) {
-                ws->ranks = (uint32_t *)device_alloc(std::max<size_t>(ws->nwords, 1) * 4);
-                ws->bytes += size_t(ws->nwords) * 4;
-            }
+            ensure_ranks(ws);
             grow(ws, &ws->hist, &ws->hist_cap, hist_words(nranks), 4);
             const uint32_t nblocks = std::max<uint32_t>((ws->nwords + 1023) / 1024, 1);
             const bool counted = nblocks > COMPACT_BLOCKS;
@@ -4950,6 +4940,43 @@ __global__ void k_set_bits_multi(const uint32_t *__restrict__ ids, const uint32_
     }
 }
 
+// Room for nq queries of `targets` S ids in all.
+static void ensure_multi(Workspace *ws, uint32_t nq, uint64_t targets) {
+    if (ws->mq_cap_q < uint64_t(nq) + 1) {
+        for (void **p : {(void **)&ws->mq_first, (void **)&ws->mq_bound, (void **)&ws->mq_soff, (void **)&ws->mq_sptr,
+                         (void **)&ws->mq_counts, (void **)&ws->mq_swap}) {
+            device_free(*p);
+            *p = nullptr;
+        }
+        ws->mq_cap_q = 0;
+        const uint64_t cap = std::max<uint64_t>(nq + 1, 64);
+        ws->mq_swap = (uint8_t *)device_alloc(cap);
+        ws->mq_first = (uint32_t *)device_alloc(cap * 4);
+        ws->mq_bound = (uint32_t *)device_alloc(cap * 4);
+        ws->mq_soff = (uint32_t *)device_alloc(cap * 4);
+        ws->mq_sptr = (const uint32_t **)device_alloc(cap * 8);
+        ws->mq_counts = (unsigned long long *)device_alloc(cap * 8);
+        ws->mq_cap_q = cap;
+    }
+    const uint64_t bits_words = uint64_t(nq) * ws->nwords;
+    if (ws->mq_cap_bits < bits_words) {
+        device_free(ws->mq_sbits);
+        ws->mq_sbits = nullptr;
+        ws->mq_cap_bits = 0;
+        const uint64_t cap = bits_words + bits_words / 2;
+        ws->mq_sbits = (uint32_t *)device_alloc(cap * 4);
+        ws->mq_cap_bits = cap;
+    }
+    if (ws->mq_cap_sids < std::max<uint64_t>(targets, 1)) {
+        device_free(ws->mq_sids);
+        ws->mq_sids = nullptr;
+        ws->mq_cap_sids = 0;
+        const uint64_t cap = std::max<uint64_t>(targets + targets / 2, 1024);
+        ws->mq_sids = (uint32_t *)device_alloc(cap * 4);
+        ws->mq_cap_sids = cap;
+    }
+}
+
 void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint32_t median_w,
                     const std::vector<uint32_t> &perm, const std::vector<const uint32_t *> &R,
                     const std::vector<uint32_t> &nR, const std::vector<const uint32_t *> &S,
@@ -5023,33 +5050,7 @@ void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg
             ranges.push_back(make_uint4(first[i] + j, std::min(tile_src, nsrc[i] - j), 0, 0));
     // device copies
     ensure_u32(&ws->rsorted, &ws->rsorted_cap, std::max<uint32_t>(total, 1));
-    if (ws->mq_cap_q < nq + 1) {
-        for (void **p : {(void **)&ws->mq_first, (void **)&ws->mq_bound, (void **)&ws->mq_soff, (void **)&ws->mq_sptr,
-                         (void **)&ws->mq_counts, (void **)&ws->mq_swap}) {
-            device_free(*p);
-            *p = nullptr;
-        }
-        ws->mq_cap_q = std::max<uint64_t>(nq + 1, 64);
-        ws->mq_swap = (uint8_t *)device_alloc(ws->mq_cap_q);
-        ws->mq_first = (uint32_t *)device_alloc(ws->mq_cap_q * 4);
-        ws->mq_bound = (uint32_t *)device_alloc(ws->mq_cap_q * 4);
-        ws->mq_soff = (uint32_t *)device_alloc(ws->mq_cap_q * 4);
-        ws->mq_sptr = (const uint32_t **)device_alloc(ws->mq_cap_q * 8);
-        ws->mq_counts = (unsigned long long *)device_alloc(ws->mq_cap_q * 8);
-    }
-    const uint64_t bits_words = uint64_t(nq) * ws->nwords;
-    if (ws->mq_cap_bits < bits_words) {
-        device_free(ws->mq_sbits);
-        ws->mq_sbits = nullptr;
-        ws->mq_cap_bits = bits_words + bits_words / 2;
-        ws->mq_sbits = (uint32_t *)device_alloc(ws->mq_cap_bits * 4);
-    }
-    if (ws->mq_cap_sids < std::max<size_t>(sids.size(), 1)) {
-        device_free(ws->mq_sids);
-        ws->mq_sids = nullptr;
-        ws->mq_cap_sids = std::max<uint64_t>(sids.size() + sids.size() / 2, 1024);
-        ws->mq_sids = (uint32_t *)device_alloc(ws->mq_cap_sids * 4);
-    }
+    ensure_multi(ws, nq, sids.size());
     std::vector<const uint32_t *> sptr(nq);
     for (uint32_t i = 0; i < nq; i++) sptr[i] = ws->mq_sbits + size_t(i) * ws->nwords;
     if (total) RN_CUDA(cudaMemcpyAsync(ws->rsorted, src.data(), size_t(total) * 4, cudaMemcpyHostToDevice, st));
@@ -5060,7 +5061,7 @@ void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg
     if (any_swap) RN_CUDA(cudaMemcpyAsync(ws->mq_swap, swp.data(), nq, cudaMemcpyHostToDevice, st));
     if (!sids.empty())
         RN_CUDA(cudaMemcpyAsync(ws->mq_sids, sids.data(), sids.size() * 4, cudaMemcpyHostToDevice, st));
-    RN_CUDA(cudaMemsetAsync(ws->mq_sbits, 0, bits_words * 4, st));
+    RN_CUDA(cudaMemsetAsync(ws->mq_sbits, 0, size_t(nq) * ws->nwords * 4, st));
     RN_CUDA(cudaMemsetAsync(ws->mq_counts, 0, size_t(nq) * 8, st));
     RN_CUDA(cudaMemsetAsync(ws->ctl, 0, sizeof(Control), st));
     if (!sids.empty()) {
@@ -5420,6 +5421,32 @@ __global__ void k_compact_le(const unsigned long long *__restrict__ kin, const u
     }
 }
 
+static void ensure_kcp(Workspace *ws) {
+    if (ws->kcp) return;
+    ws->kcp = (uint32_t *)device_alloc((KCP_BINS + 16) * 4 + sizeof(SelState));
+    ws->bytes += (KCP_BINS + 16) * 4 + sizeof(SelState);
+}
+
+// Grow the workspace's buffers now for queries of up to max_r sources and max_pairs pairs (raw
+// pairs and their sort), and for joins searched together of up to max_queries queries and
+// max_targets targets in all, so that such queries allocate and free nothing later (but the tile
+// search's maps in device memory): freeing device memory synchronises the whole device, which
+// would stall every other stream's work.
+void workspace_reserve(Workspace *ws, uint32_t max_r, uint64_t max_pairs, uint32_t max_queries, uint64_t max_targets) {
+    ensure_u32(&ws->rsorted, &ws->rsorted_cap, std::max<uint32_t>(max_r, 1));
+    ensure_ranges(&ws->failed, &ws->failed_cap, std::max<uint32_t>(max_r, 1));
+    ensure_ranges(&ws->failed2, &ws->failed2_cap, std::max<uint32_t>(max_r, 1));
+    ensure_pairs(ws, max_pairs);
+    grow(ws, &ws->hist, &ws->hist_cap, sort_words(max_pairs), 4);
+    ensure_slist(ws);
+    ensure_segments(ws, max_r);
+    ensure_ranks(ws);
+    ensure_kcp(ws);
+    ensure_multi(ws, max_queries, max_targets);
+    ensure_place_state(ws, (max_r + PLACE_SEGS - 1) / PLACE_SEGS, nullptr);
+    RN_CUDA(cudaDeviceSynchronize());  // before any query on a stream of its own
+}
+
 void run_kcp(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint32_t median_w, const uint32_t *dR,
              uint32_t nR, const uint32_t *dS, uint32_t nS, uint64_t k, uint32_t theta, rn_dpairs *out, void *stream,
              rn_query_stats *stats) {
@@ -5453,10 +5480,7 @@ void run_kcp(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint3
     ensure_ranges(&ws->failed, &ws->failed_cap, std::max<uint32_t>(std::max(ntiles, nR), 1));
     ensure_ranges(&ws->failed2, &ws->failed2_cap, std::max<uint32_t>(std::max(ntiles, nR), 1));
     ensure_pairs(ws, std::max<uint64_t>(ws->pair_cap, std::min<uint64_t>(k + (k >> 2) + 4096, uint64_t(nR) * 64 + 4096)));
-    if (!ws->kcp) {
-        ws->kcp = (uint32_t *)device_alloc((KCP_BINS + 16) * 4 + sizeof(SelState));
-        ws->bytes += (KCP_BINS + 16) * 4 + sizeof(SelState);
-    }
+    ensure_kcp(ws);
     uint32_t *hist = ws->kcp, *theta_live = ws->kcp + KCP_BINS;
     SelState *sel = reinterpret_cast<SelState *>(ws->kcp + KCP_BINS + 16);
 

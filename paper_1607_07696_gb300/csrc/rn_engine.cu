@@ -101,6 +101,16 @@ void *device_alloc(size_t bytes) {
     return p;
 }
 
+// The same, or null where there is not enough memory.
+static void *device_try_alloc(size_t bytes) {
+    try {
+        return device_alloc(bytes);
+    } catch (const Error &e) {
+        if (e.status != RN_ENOMEM) throw;
+        return nullptr;
+    }
+}
+
 void device_free(void *p) {
     if (!p) return;
     Hook h;
@@ -4169,16 +4179,21 @@ static void build_rows(const HostGraph &g, DeviceGraph *d) {
     d->far = g.n ? uint64_t(g.n - 1) * max_w : 0;
     d->paged = max_deg <= 64 && 5 * inside >= 2 * g.arcs() && 4 * nvirt <= 3 * uint64_t(g.n) && g.n + nvirt <= PG_ROWS_MAX;
     if (!d->paged) return;
+    d->ell = (uint4 *)device_try_alloc(std::max<uint64_t>(g.n + nvirt, 1) * PG_ROW * 8);
+    uint2 *dh = heavy.empty() || !d->ell ? nullptr : (uint2 *)device_try_alloc(heavy.size() * 8);
+    if (!d->ell || (!heavy.empty() && !dh)) {  // no room for the rows: the hashed search needs none
+        device_free(d->ell);
+        d->ell = nullptr;
+        d->paged = false;
+        return;
+    }
     d->nvirt = uint32_t(nvirt);
     d->row_chain = max_deg <= PG_ROW ? 0 : (max_deg - PG_ROW + PG_ROW - 2) / (PG_ROW - 1);
-    d->ell = (uint4 *)device_alloc(std::max<uint64_t>(g.n + nvirt, 1) * PG_ROW * 8);
     uint2 *rows = reinterpret_cast<uint2 *>(d->ell);
     const uint2 *adj = reinterpret_cast<const uint2 *>(d->adj);
     if (g.n) k_rows<<<rows_grid(uint64_t(g.n) * PG_ROW), 256>>>(d->row_ptr, adj, g.n, rows);
     RN_CUDA(cudaGetLastError());
-    uint2 *dh = nullptr;
-    if (!heavy.empty()) {
-        dh = (uint2 *)device_alloc(heavy.size() * 8);
+    if (dh) {
         const cudaError_t e = cudaMemcpy(dh, heavy.data(), heavy.size() * 8, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) {
             const uint32_t count = uint32_t(heavy.size());
@@ -5903,19 +5918,19 @@ static void points_graph(const DeviceGraph &g, const std::vector<uint32_t> &perm
         ps->aug.adj = (uint32_t *)device_alloc(cap_arcs * 8);
         ps->aug.perm = (uint32_t *)device_alloc(cap_nodes * 4);
         ps->aug.iperm = (uint32_t *)device_alloc(cap_nodes * 4);
-        if (g.paged) ps->aug.ell = (uint4 *)device_alloc((cap_nodes + g.nvirt) * PG_ROW * 8);
         workspace_destroy(ps->ws);
         ps->ws = nullptr;
         DeviceGraph capg{};
         capg.n = uint32_t(cap_nodes);
         ps->ws = workspace_create(capg);
+        if (g.paged) ps->aug.ell = (uint4 *)device_try_alloc((cap_nodes + g.nvirt) * PG_ROW * 8);
         ps->cap_nodes = cap_nodes;
         ps->cap_arcs = cap_arcs;
     }
     ps->aug.n = uint32_t(n_aug);
     ps->aug.arcs = arcs_aug;
     ps->aug.nvirt = g.nvirt;
-    ps->aug.paged = g.paged && n_aug + g.nvirt <= PG_ROWS_MAX;
+    ps->aug.paged = g.paged && ps->aug.ell && n_aug + g.nvirt <= PG_ROWS_MAX;
     ps->aug.far = g.far;  // (a path crosses an edge's links at most once: no longer than over whole edges)
     // staged: links (4 words a point), output ids, node of every point (R's then S's), patches
     std::memcpy(ps->host, tail.data(), size_t(np) * 16);
@@ -7522,6 +7537,10 @@ Batch *batch_create(const std::vector<const DeviceGraph *> &graphs, const std::v
             vsum += graphs[i]->nvirt;
         }
         b->paged = b->paged && nsum + 1 + vsum <= PG_ROWS_MAX && (b->theta_max <= PG_BOUND_MAX || b->ug.far <= PG_BOUND_MAX);
+        if (b->paged) {
+            b->ug.ell = (uint4 *)device_try_alloc((nsum + 1 + vsum) * PG_ROW * 8);
+            b->paged = b->ug.ell != nullptr;
+        }
         nsum = 0;
         for (uint32_t i = 0; i < b->nq; i++) {
             b->n[i] = graphs[i]->n;
@@ -7566,7 +7585,6 @@ Batch *batch_create(const std::vector<const DeviceGraph *> &graphs, const std::v
         if (b->paged) {
             b->ug.paged = true;
             b->ug.nvirt = uint32_t(vsum);
-            b->ug.ell = (uint4 *)device_alloc((size_t(b->n_u) + vsum) * PG_ROW * 8);
             uint64_t voff = b->n_u;
             for (uint32_t i = 0; i < b->nq; i++) {
                 const DeviceGraph &g = *graphs[i];

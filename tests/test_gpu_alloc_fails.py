@@ -99,3 +99,42 @@ def test_every_allocation_fails_once(rn, world, kind):
             for run in range(2):
                 assert same(call(g), ref), (nth, run)
         assert not a.refused and failed >= 5
+
+
+def test_without_room_for_rows(rn, world, oracle):
+    """The rows of the search by pages are extra memory (64 bytes a node and overflow row): graphs,
+    points and batches for which they do not fit are answered by the hashed search."""
+    e, og, med = world
+    deg = np.bincount(np.r_[e.src, e.dst], minlength=e.n)  # (no loops or parallel edges)
+    rows = int(((np.maximum(deg, 8) - 8 + 6) // 7).sum())
+    R, S = I.disjoint_sets(e.n, 700, 900, 224)
+    ref, refk = og.join(R, S, 12 * med), og.kcp(R, S, 3_000)
+    pts = pins.random_points(np.random.default_rng(225), pins.least_weights(e), 900)
+    refp = og.join_points(pts[:400], pts[400:], 12 * med)
+
+    def answers(g):
+        for run in range(2):
+            assert same(rn.rn_distance_join(g, R, S, 12 * med), ref), run
+            assert same(rn.rn_kcp(g, R, S, 3_000), refk), run
+            assert same(rn.rn_distance_join_points(g, pts[:400], pts[400:], 12 * med), refp), run
+            assert same(rn.rn_distance_join_hier(g, R, S, 12 * med, 2048), ref), run
+
+    def batch(g):
+        b = rn.rn_batch_create([(g, R, S, 12 * med), (g, S[:80], R, 5 * med)])
+        for run in range(4):  # eager, laid out again, recorded, replayed
+            rn.rn_batch_run(b)
+            assert same(rn.rn_batch_pairs(b, 0), ref) and same(rn.rn_batch_pairs(b, 1), og.join(S[:80], R, 5 * med)), run
+
+    with Allocator(rn) as a:
+        a.sizes = (64 * (e.n + rows),)
+        g = rn.rn_graph_load(e.src, e.dst, e.w, e.n)
+        assert a.refused == [64 * (e.n + rows)]
+        a.sizes = ()
+        answers(g)
+        batch(g)
+        g = rn.rn_graph_load(e.src, e.dst, e.w, e.n)
+        n = e.n + 900
+        a.sizes, a.refused = (64 * (n + n // 4 + rows), 64 * (2 * e.n + 1 + 2 * rows)), []  # points', a batch's
+        answers(g)
+        batch(g)
+        assert a.refused == list(a.sizes)

@@ -6255,9 +6255,9 @@ __global__ void k_exit_flags(const unsigned long long *__restrict__ key, uint64_
     }
 }
 
-// Compact the kept exit routes (each (f, si) with its least offset: records sorted by key
-// then offset) into (j << 32 | si, off), j the index of far end f in f_list; f_list[j] =
-// orig(f), fmin[j] = its least offset (fmin starts at INF).
+// Compact the kept exit routes (each (f, si) with its least offset, found over its run: the
+// records are sorted by key alone) into (j << 32 | si, off), j the index of far end f in
+// f_list; f_list[j] = orig(f), fmin[j] = its least offset (fmin starts at INF).
 __global__ void k_exit_compact(const unsigned long long *__restrict__ key, const uint32_t *__restrict__ d, uint64_t m,
                                const uint32_t *__restrict__ keep, const uint32_t *__restrict__ keep_at,
                                const uint32_t *__restrict__ head, const uint32_t *__restrict__ head_at,
@@ -6267,7 +6267,11 @@ __global__ void k_exit_compact(const unsigned long long *__restrict__ key, const
         const unsigned long long k = key[i];
         const uint32_t j = head_at[i] + head[i] - 1;
         if (head[i]) f_list[j] = uint32_t(k >> 32);
-        uint32_t least = d[i];  // (a run of equal keys, one or two long, is in no order of distance)
+        // A run of equal keys holds an offset, in no order, for every arc from the source's part into f
+        // that the source reaches: mostly one or two, and one thread reads it.  (With 15,000 arcs into
+        // one node, 3,000 sources, no bound, parts of 2,048 / 4,096 nodes, the call takes 110 / 112 ms;
+        // with the offsets among the sort's digits and hashed searches it had taken 114 / 117)
+        uint32_t least = d[i];
         for (uint64_t r = i + 1; r < m && key[r] == k; r++) least = min(least, d[r]);
         e_key[keep_at[i]] = ((unsigned long long)j << 32) | uint32_t(k);
         e_off[keep_at[i]] = least;
@@ -6363,20 +6367,20 @@ __global__ void k_hier_combine(const unsigned long long *__restrict__ e_key, con
     }
 }
 
-// Flags of the first record of every key (records sorted by key, then distance).
+// Flags of the first record of every key (records sorted by key).
 __global__ void k_first_of_key(const unsigned long long *__restrict__ key, uint64_t m, uint32_t *first) {
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < m; i += uint64_t(gridDim.x) * blockDim.x)
         first[i] = i == 0 || key[i - 1] != key[i];
 }
 
-// The first (least-distance) record of every key, compacted in key order.
+// Every key with its least distance, compacted in key order.
 __global__ void k_first_compact(const unsigned long long *__restrict__ key, const uint32_t *__restrict__ d, uint64_t m,
                                 const uint32_t *__restrict__ first, const uint32_t *__restrict__ at,
                                 unsigned long long *okey, uint32_t *od) {
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < m; i += uint64_t(gridDim.x) * blockDim.x) {
         if (!first[i]) continue;
         const unsigned long long k = key[i];
-        uint32_t least = d[i];  // (a run of equal keys is in no order of distance)
+        uint32_t least = d[i];  // (a run holds a candidate for every exit route that reaches v, in no order)
         for (uint64_t r = i + 1; r < m && key[r] == k; r++) least = min(least, d[r]);
         okey[at[i]] = k;
         od[at[i]] = least;
@@ -6684,7 +6688,7 @@ void run_hier(const DeviceGraph &g, Workspace *ws, HierState **state, const Engi
         late_check(ws);  // (the sort of the hits, before they are used)
         mark();
         // 4. candidates through the exit arcs after the local pairs, then every pair's least
-        // distance (records sorted by (u, v) and distance; the first of each (u, v) kept)
+        // distance (records sorted by (u, v); the least of each run kept)
         uint64_t cap = std::max<uint64_t>({local + nh * 2, h->candidates + h->candidates / 8, 1 << 16}), m = 0;
         unsigned long long *mk0 = nullptr;
         uint32_t *md0 = nullptr;

@@ -83,3 +83,20 @@ def test_parts_of_overflow_rows(rn, oracle, size, hub, part):
         assert same(rn.rn_distance_join_hier(g, R, S, theta, part), ref), theta
         assert part / 2 < rn.rn_last_hier_stats()["max_part"] <= part
     assert same(rn.rn_kcp_hier(g, R, S, 2_000, rn.RN_INF, part), og.kcp(R, S, 2_000))
+
+
+@pytest.mark.parametrize("part", [512, 4096])
+def test_many_arcs_into_one_node(rn, oracle, part):
+    """A node that hundreds of arcs of every part lead to: each source has as many routes to it,
+    of which the least counts."""
+    e = I.road_graph(8_000, 20_800, 231)
+    rng = np.random.default_rng(232)
+    t = rng.choice(np.arange(1, e.n), 5_000, replace=False)
+    e = I.EdgeList(e.n, np.r_[e.src, e.dst, t].astype(np.uint32), np.r_[e.dst, e.src, np.zeros(len(t))].astype(np.uint32),
+                   np.r_[e.w, e.w, rng.integers(1, 3_000, len(t))].astype(np.uint32), None, {})
+    g = rn.rn_graph_load(e.src, e.dst, e.w, e.n, flags=rn.RN_REORDER)
+    og = oracle.graph(e.n, e.src, e.dst, e.w, undirected=False)
+    R, S = I.disjoint_sets(e.n, 600, 200, 233)
+    for theta in (8_000, rn.RN_INF):
+        ref = og.join(R, S, min(theta, rn.RN_THETA_MAX))
+        assert same(rn.rn_distance_join_hier(g, R, S, theta, part), ref), theta

@@ -70,7 +70,8 @@ struct DeviceGraph {
     bool symmetric = false;          // every arc has its reverse with the same weight (undirected)
     // the source search's rows: eight arc slots (col, w) per node, a node with more arcs
     // going on in overflow rows n, n + 1, ... (nvirt of them; at most row_chain per node);
-    // paged: the ids have the locality the search by pages wants; far: no distance is longer
+    // paged: the ids have the locality the search by pages wants, and the rows are there; far:
+    // no distance is longer
     uint4 *ell = nullptr;
     uint32_t nvirt = 0, row_chain = 0;
     bool paged = false;

@@ -1990,8 +1990,8 @@ __global__ void __launch_bounds__(32 * W * pg_groups(W), 32 / (W * pg_groups(W))
 
 // ----------------------------------------------------- hashed source search ----
 // The search of graphs whose node ids carry no locality (loaded without the bisection
-// order, or with hubs), where a page would hold a node or two, and of graphs of many overflow
-// rows (build_rows) or without room for rows: the ball's nodes are hashed one by one.
+// order, or with hubs), where a page would hold a node or two: the ball's nodes are hashed
+// one by one.
 //
 // One warp searches one source at a time (persistent: warps pop sources from the work
 // counter).  The source's ball lives in a map of MS slots in shared memory that only this

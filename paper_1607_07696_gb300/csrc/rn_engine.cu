@@ -7077,7 +7077,7 @@ static bool batch_adapt_maps(Batch *b) {
 
 // Group the instances by (tile width, first map, sources per tile) and upload each
 // group's padded source list and per-tile tables.
-static void batch_layout(Batch *b) {
+static void batch_layout_groups(Batch *b) {
     batch_drop_graph(b);
     batch_free_groups(b);
     std::map<std::tuple<uint32_t, uint32_t, uint32_t>, std::vector<uint32_t>> by;
@@ -7122,12 +7122,13 @@ static void batch_layout(Batch *b) {
             if (x >= b->n_u) fail(RN_EINTERNAL, "batch layout: source outside the union graph");
         g.nsrc = uint32_t(src.size());
         g.tiles = uint32_t(tb.size());
-        g.src = upload_vec(src);
-        g.tbound = upload_vec(tb);
-        g.tdelta = upload_vec(td);
-        g.tinst = upload_vec(ti);
         tiles += g.tiles;
         b->groups.push_back(g);
+        Batch::Group &kept = b->groups.back();  // (freed with the others if an upload fails)
+        kept.src = upload_vec(src);
+        kept.tbound = upload_vec(tb);
+        kept.tdelta = upload_vec(td);
+        kept.tinst = upload_vec(ti);
     }
     RN_CUDA(cudaDeviceSynchronize());  // the batch's stream does not wait for these copies
     ensure_ranges(&b->ws->failed, &b->ws->failed_cap, uint32_t(std::max<uint64_t>(tiles, 1)));
@@ -7136,9 +7137,20 @@ static void batch_layout(Batch *b) {
     b->stats.groups = uint32_t(b->groups.size());
 }
 
+// A layout that fails half way leaves no group, and the next run makes it again.
+static void batch_layout(Batch *b) {
+    try {
+        batch_layout_groups(b);
+    } catch (...) {
+        batch_free_groups(b);
+        throw;
+    }
+}
+
 static void batch_reserve_pairs(Batch *b, uint64_t want) {
     if (b->pair_cap >= want) return;
     want = std::max<uint64_t>(want, 1 << 16);
+    batch_drop_graph(b);
     for (void **p : {(void **)&b->keyA, (void **)&b->keyB, (void **)&b->valA, (void **)&b->valB}) {
         device_free(*p);
         *p = nullptr;
@@ -7149,7 +7161,6 @@ static void batch_reserve_pairs(Batch *b, uint64_t want) {
     b->valA = (uint32_t *)device_alloc(want * 4);
     b->valB = (uint32_t *)device_alloc(want * 4);
     b->pair_cap = want;
-    batch_drop_graph(b);
 }
 
 static SearchArgs batch_args(Batch *b, const Batch::Group &g) {
@@ -7266,6 +7277,8 @@ static void batch_launch_group(Batch *b, const Batch::Group &g, cudaStream_t st,
 // the pair buffer.  Returns the number of retried tiles.
 static uint64_t batch_run_eager(Batch *b, cudaStream_t st) {
     b->ws->own_gmap_moved = false;
+    if (b->groups.empty()) batch_layout(b);  // (its last layout failed)
+    batch_reserve_pairs(b, 1);
     for (;;) {
         batch_clear(b, st);
         uint64_t retried = 0;

@@ -138,3 +138,32 @@ def test_without_room_for_rows(rn, world, oracle):
         answers(g)
         batch(g)
         assert a.refused == list(a.sizes)
+
+
+def test_every_allocation_of_a_batch_fails_once(rn, world):
+    """Balls past the first maps, so that the batch is laid out again between its runs."""
+    e, og, med = world
+    R, S = I.disjoint_sets(e.n, 500, 600, 226)
+    queries = [(R, S, 45 * med), (S[:90], R, 5 * med), (R[:200], S[:300], 20 * med)]
+    refs = [og.join(*q) for q in queries]
+    g = rn.rn_graph_load(e.src, e.dst, e.w, e.n)
+    with Allocator(rn) as a:
+        failed = 0
+        for nth in range(1, 200):
+            b = rn.rn_batch_create([(g, *q) for q in queries])
+            a.left, a.refused = nth, []
+            for run in range(4):  # eager, laid out again, recorded, replayed
+                try:
+                    rn.rn_batch_run(b)
+                except rn.RNError as ex:
+                    assert ex.status == rn.RN_ENOMEM, (nth, ex)
+                    failed += 1
+                    break
+                assert all(same(rn.rn_batch_pairs(b, i), ref) for i, ref in enumerate(refs)), (nth, run)
+            a.left = None
+            if not a.refused:
+                break
+            for run in range(4):
+                rn.rn_batch_run(b)
+                assert all(same(rn.rn_batch_pairs(b, i), ref) for i, ref in enumerate(refs)), (nth, run)
+        assert not a.refused and failed >= 8
